@@ -10,11 +10,10 @@
 //   4. scatter: one CTA per chunk: write the masks, a 128-row prefix sum of the
 //               popcounts gives each row's first value slot, rows copy their kept
 //               values in ascending column order, and the padding is zeroed.
-// sp_decompress is the inverse (one CTA per chunk, one thread per row).
-// None of this is on the timed path.
+// sp_decompress is the inverse (described at its kernel).
 #include <algorithm>
 
-#include "sp_internal.cuh"
+#include "sp_expand.cuh"
 
 namespace sp {
 namespace {
@@ -166,33 +165,101 @@ __global__ void __launch_bounds__(kRows) scatter_kernel(const uint8_t* __restric
   for (uint64_t b = used + r; b < size; b += kRows) chunk[b] = 0;
 }
 
+// Dense masked weight from the compressed form.  Bound by memory: the compressed bytes in,
+// N * K * ES bytes out, so the kernel is laid out for the dense stores.  One CTA of four
+// warps per chunk: one bulk copy brings the chunk to shared memory, warp q expands rows
+// 32q .. 32q+31 on its own (the quarter index gives its first value, one warp scan the start
+// of each 32-column half row), and a lane expands 16 bytes of one row, so a warp stores
+// whole 64 * ES byte row segments, 16 bytes per lane.  One thread per row storing its 64
+// columns two bytes at a time touched 32 rows per store.  Measured, 22016 x 4096 bf16 at 70 %:
+// 654 -> 39.1 us (245 MB in and out, 6.3 TB/s).
+template <int ES>
 __global__ void __launch_bounds__(kRows) decompress_kernel(const uint8_t* __restrict__ buf,
-                                                           const uint64_t* __restrict__ off, int esize, int64_t N,
-                                                           int64_t K, int T, uint8_t* __restrict__ out) {
-  __shared__ int s_warp[kRows / 32];
+                                                           const uint64_t* __restrict__ off,
+                                                           const uint64_t* __restrict__ qidx, int64_t N, int64_t K,
+                                                           int T, uint8_t* __restrict__ out, uint64_t timeout_ns,
+                                                           int* status) {
+  extern __shared__ __align__(128) uint8_t chunk[];
+  __shared__ uint64_t bar;
+  __shared__ uint32_t s_start[2 * kRows];  // byte offset of each 32-column half row's first value
+  constexpr int kCols = 16 / ES;           // columns per lane
+  constexpr int kSegs = kTileK / kCols;    // lanes per row
   const int64_t c = blockIdx.x;
   const int64_t rb = c / T, t = c % T;
-  const int r = threadIdx.x;
-  const int64_t n = rb * kRows + r;
-  const uint8_t* chunk = buf + off[c];
-  const uint64_t m = reinterpret_cast<const uint64_t*>(chunk)[r];
-  int total;
-  const int e0 = block_excl_scan_128(__popcll(m), &total, s_warp);
-  if (n >= N) return;
-  const uint8_t* vals = chunk + kMaskBytes;
-  const int valid = (int)imin64((int64_t)kTileK, K - (int64_t)kTileK * t);
-  uint8_t* row = out + (n * K + (int64_t)kTileK * t) * esize;
-  int i = 0;
-  for (int j = 0; j < valid; ++j) {
-    const bool kept = (m >> j) & 1u;
-    if (esize == 2) {
-      uint16_t v = 0;
-      if (kept) v = *reinterpret_cast<const uint16_t*>(vals + 2 * (e0 + i));
-      reinterpret_cast<uint16_t*>(row)[j] = v;
-    } else {
-      row[j] = kept ? vals[e0 + i] : 0;
+  const int tid = threadIdx.x, lane = tid & 31, q = tid >> 5;
+  if (tid == 0) {
+    mbar_init(&bar, 1);
+    fence_barrier_init();
+    const uint64_t o0 = off[c];
+    const uint32_t bytes = (uint32_t)(off[c + 1] - o0);
+    mbar_arrive_expect_tx(&bar, bytes);
+    bulk_g2s(chunk, buf + o0, bytes, &bar);
+  }
+  const uint64_t qi = qidx[c];
+  __syncthreads();
+  if (!__all_sync(0xffffffffu, mbar_wait(&bar, 0, timeout_ns))) {
+    set_status(status, kStatusTimeout);
+    return;
+  }
+  const uint32_t* words = reinterpret_cast<const uint32_t*>(chunk);  // word 2r, 2r + 1: row r's mask
+  {
+    const uint2 m = reinterpret_cast<const uint2*>(chunk)[tid];
+    const int plo = __popc(m.x), pc = plo + __popc(m.y);
+    int incl = pc;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += u;
     }
-    i += kept;
+    const int before = q == 0 ? 0 : (int)((qi >> (16 * (q - 1))) & 0xffffu);
+    const uint32_t e0 = (uint32_t)(before + incl - pc);
+    reinterpret_cast<uint2*>(s_start)[tid] = make_uint2(e0 * ES, (e0 + (uint32_t)plo) * ES);
+  }
+  __syncwarp();
+  const int seg = lane % kSegs;
+  const int half = seg / (kSegs / 2);                 // which mask word holds the lane's columns
+  const int sh = kCols * (seg % (kSegs / 2));         // and where they start in it
+  const uint32_t below = (1u << sh) - 1u;
+  const uint32_t vbase = smem_u32(chunk) + kMaskBytes;
+  const int64_t col = (int64_t)kTileK * t + kCols * seg;
+  const int64_t pitch = K * ES;
+  uint8_t* dst = out + (rb * kRows + 32 * q + lane / kSegs) * pitch + col * ES;
+#pragma unroll 2
+  for (int i = 0; i < kSegs; ++i) {  // 32 / kSegs rows at a time
+    const int r = 32 * q + i * (32 / kSegs) + lane / kSegs;
+    const uint32_t w = words[2 * r + half];
+    uint32_t pa = vbase + s_start[2 * r + half] + (uint32_t)(ES * __popc(w & below));
+    const uint32_t m = w >> sh;
+    uint4 o;
+    if constexpr (ES == 2) {
+      o.x = expand_word_bf16<1u, 2u>(m, pa);
+      o.y = expand_word_bf16<4u, 8u>(m, pa);
+      o.z = expand_word_bf16<16u, 32u>(m, pa);
+      o.w = expand_word_bf16<64u, 128u>(m, pa);
+    } else {
+      uint32_t a[8];
+      a[0] = expand_word_u8<1u << 0, 1u << 1>(m, pa);
+      a[1] = expand_word_u8<1u << 2, 1u << 3>(m, pa);
+      a[2] = expand_word_u8<1u << 4, 1u << 5>(m, pa);
+      a[3] = expand_word_u8<1u << 6, 1u << 7>(m, pa);
+      a[4] = expand_word_u8<1u << 8, 1u << 9>(m, pa);
+      a[5] = expand_word_u8<1u << 10, 1u << 11>(m, pa);
+      a[6] = expand_word_u8<1u << 12, 1u << 13>(m, pa);
+      a[7] = expand_word_u8<1u << 14, 1u << 15>(m, pa);
+      o = make_uint4(__byte_perm(a[0], a[1], 0x6420), __byte_perm(a[2], a[3], 0x6420),
+                     __byte_perm(a[4], a[5], 0x6420), __byte_perm(a[6], a[7], 0x6420));
+    }
+    if (rb * kRows + r < N && col < K) {
+      // K % 8 == 0: a bf16 row's segments are whole and 16-byte aligned; an int8 row starts
+      // on an 8-byte boundary and its last segment may hold 8 columns
+      if (ES == 2 || K % 16 == 0) {
+        __stcs(reinterpret_cast<uint4*>(dst), o);
+      } else {
+        __stcs(reinterpret_cast<uint2*>(dst), make_uint2(o.x, o.y));
+        if (col + 8 < K) __stcs(reinterpret_cast<uint2*>(dst + 8), make_uint2(o.z, o.w));
+      }
+    }
+    dst += (int64_t)(32 / kSegs) * pitch;
   }
 }
 
@@ -312,8 +379,10 @@ fail:
 
 sp_status launch_decompress(const sp_matrix* h, void* w_out, cudaStream_t stream) {
   const int64_t C = (int64_t)h->RB * h->T;
-  decompress_kernel<<<(unsigned)C, kRows, 0, stream>>>(h->d_buf, h->d_off, h->esize, h->N, h->K, h->T,
-                                                        (uint8_t*)w_out);
+  const size_t smem = (size_t)h->max_chunk;  // at most 1024 + 128 * 64 * 2 bytes
+  auto kern = h->esize == 2 ? decompress_kernel<2> : decompress_kernel<1>;
+  kern<<<(unsigned)C, kRows, smem, stream>>>(h->d_buf, h->d_off, h->d_qidx, h->N, h->K, h->T, (uint8_t*)w_out,
+                                             wait_timeout_ns(), device_status_ptr());
   return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ERR_CUDA;
 }
 
