@@ -163,3 +163,25 @@ def test_argument_errors(sp):
     hi = sp.compress(gu.i8_to_dev(q), gu.u8_to_dev(mask), gu.f32_to_dev(s))
     assert lib.sp_masked_update(hi.handle, ctypes.c_void_p(gd.data_ptr()), ctypes.c_float(0.1), None) == 2
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("N,K", [(130, 72), (129, 4096)])
+def test_gradient_on_a_16_byte_boundary(sp, oracle, N, K):
+    """The kernel takes 32-byte gradient loads only where the pointer is 32-byte aligned; a
+    gradient that starts 16 bytes later gives the same bytes."""
+    import torch
+
+    g = np.random.default_rng(N)
+    W = synth.weight(N, K, g)
+    mask = synth.magnitude_mask(W, 60)
+    grad = g.standard_normal((N, K), dtype=np.float32)
+    flat = torch.zeros(N * K + 4, dtype=torch.float32, device=gu.dev())
+    gd = flat[4:].view(N, K)
+    gd.copy_(torch.from_numpy(grad))
+    assert flat.data_ptr() % 32 == 0 and gd.data_ptr() % 32 == 16
+    h = sp.compress(gu.bf16_to_dev(W), gu.u8_to_dev(mask))
+    h.masked_update(gd, 0.01)
+    sp.check()
+    buf, _ = h.copy_out()
+    obuf, ooff = oracle.compress(W, mask)
+    assert np.array_equal(buf, oracle.masked_update_bf16(obuf, ooff, N, K, grad, 0.01))
