@@ -64,8 +64,7 @@ typedef enum sp_status {
 typedef enum sp_dtype { SP_BF16 = 0, SP_INT8 = 1 } sp_dtype;
 
 /* Kernel family used by sp_linear_ex.  SP_PATH_AUTO picks by batch size M: the CUDA-core
-   family for M <= 10 (bf16 values) or M <= 13 (int8 values), the tensor-core family above
-   (the measured crossover on the Llama-2-7B shapes). */
+   family for M <= 10 (bf16 values) or M <= 13 (int8 values), the tensor-core family above. */
 typedef enum sp_path {
   SP_PATH_AUTO = 0,
   SP_PATH_CUDA_CORE = 1,    /* popc-prefix expansion, FP32 FMA on CUDA cores */
@@ -133,7 +132,10 @@ sp_status sp_linear(const sp_matrix* h, const void* x_dev, int64_t m, void* y_de
 sp_status sp_linear_ex(const sp_matrix* h, const void* x_dev, int64_t m, void* y_dev, void* workspace_dev,
                        size_t workspace_bytes, sp_path path, void* stream);
 
-/* Kernels that sp_linear_ex can launch (reported by sp_launch_count). */
+/* Kernels that sp_linear_ex can launch (reported by sp_launch_count): the family's choice for
+   the batch.  Within either family, batches of 2 .. 32 rows mostly run on linear_mma_kernel
+   (warp-level matrix instructions on chunks expanded in registers), which is the faster one
+   there; the report stays the family's. */
 enum {
   SP_KERNEL_NONE = 0,
   SP_KERNEL_CC_THREAD_PER_ROW = 1,  /* linear_cc_kernel: four warps share a chunk, thread = row */

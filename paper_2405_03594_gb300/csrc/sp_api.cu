@@ -22,11 +22,10 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 bool live(const sp_matrix* h) { return h && h->magic == SP_MAGIC; }
 
-// Largest batch that the CUDA-core family takes under SP_PATH_AUTO; larger batches go
-// to the tensor-core family.  Measured crossover on the Llama-2-7B shapes at 70%: the
-// CUDA-core path costs ~M FMAs per kept weight and the tensor-core path a fixed
-// expansion per chunk, so the tensor cores win from M ~ 11 (bf16 values) and from
-// M ~ 14 (int8 values, whose CUDA-core loop is cheaper and whose expansion costs more).
+// Largest batch that the CUDA-core family takes under SP_PATH_AUTO, and that sp_linear_epi
+// accepts; larger batches go to the tensor-core family.  The line was the crossover of
+// linear_cc_kernel and linear_tc_kernel; both families now run linear_mma_kernel around it, so
+// it only says up to which batch the epilogues of sp_chain_epilogue are available.
 constexpr int64_t kCudaCoreMaxM_bf16 = 10;
 constexpr int64_t kCudaCoreMaxM_int8 = 13;
 

@@ -296,6 +296,12 @@ sp_status launch_linear_cc(const sp_matrix* h, const uint16_t* x, int64_t M, uin
                            const uint16_t* r = nullptr);
 size_t workspace_bytes_cc(const sp_matrix* h, int64_t M);
 int cc_kernel_kind(const sp_matrix* h, int64_t M);  // 0 thread-per-row, 1 warp-per-chunk, -1 none fits
+// Batches of two to kMmaMaxRows rows on warp-level matrix instructions (no workspace); beyond,
+// the expansion is worth sharing across a wider token tile.
+constexpr int kMmaMaxRows = 32;
+bool uses_mma(const sp_matrix* h, int64_t M);  // the rule: that kernel is the faster one, and fits
+sp_status launch_linear_mma(const sp_matrix* h, const uint16_t* x, int64_t M, uint16_t* y, cudaStream_t stream,
+                            int32_t epi, const uint16_t* r);
 sp_status launch_linear_tc(const sp_matrix* h, const uint16_t* x, int64_t M, uint16_t* y, void* ws, size_t ws_bytes,
                            cudaStream_t stream);
 size_t workspace_bytes_tc(const sp_matrix* h, int64_t M);

@@ -5,11 +5,15 @@
 // memory onto the chip and are expanded there by their bitmask; decode is bound
 // by those bytes, Sec. 2.4, 3.4).
 //
-// Launch: each row block split over the S CTAs of a thread-block cluster (partials summed
-// over distributed shared memory), or -- when not even two CTAs per row block fit -- G
-// CTAs each owning a contiguous run of chunks in storage order (stream-K), so every CTA
-// streams one linear byte range.  Four CTAs per SM, six for one-row warp-per-chunk
-// cluster launches (cluster_cc and select_cc below).
+// sp_linear runs these kernels for one row, and for two rows of a large matrix; other batches
+// of up to 32 rows go to linear_mma_kernel (sp_linear_mma.cu).  More rows run here for the
+// no-allocation entry point and the failure-path test.
+//
+// Launch: each row block split over the S CTAs of a thread-block cluster (up to two rows;
+// partials summed over distributed shared memory), or -- more rows, or when not even two CTAs
+// per row block fit -- G CTAs each owning a contiguous run of chunks in storage order
+// (stream-K), so every CTA streams one linear byte range.  Four CTAs per SM, six for one-row
+// warp-per-chunk cluster launches (cluster_cc and select_cc below).
 //   warp 4, lane 0   producer: one cp.async.bulk per chunk (+ one copy of
 //                    x[m, 64t : 64t+64) per batch row) into a ring of `slots`
 //                    shared-memory slots, each guarded by a full/empty mbarrier
@@ -706,26 +710,45 @@ __global__ void __launch_bounds__(kThreads, OCC) linear_ccw_kernel(const LinearP
 template <int M, int ES>
 sp_status launch_one(const LinearParams& p, cudaStream_t stream, size_t smem, int kind, int occ, bool pdl) {
   void (*kern)(const LinearParams);
-  if constexpr (M <= 4) {
-    if (occ == kCtasPerSmM1 || occ == kCtasPerSmM1b) {
-      if constexpr (M == 1) {
-        if (kind != 1 || p.cluster < 2 || p.probe_ns != 0) return SP_ERR_UNSUPPORTED;
-        kern = occ == kCtasPerSmM1 ? linear_ccw_kernel<1, ES, true, false, kCtasPerSmM1>
-                                   : linear_ccw_kernel<1, ES, true, false, kCtasPerSmM1b>;
-      } else {
-        return SP_ERR_UNSUPPORTED;
-      }
+  if constexpr (M == 1) {
+    if (p.cluster > 1 && p.probe_ns == 0 && kind == 1) {
+      kern = occ == kCtasPerSmM1    ? linear_ccw_kernel<1, ES, true, false, kCtasPerSmM1>
+             : occ == kCtasPerSmM1b ? linear_ccw_kernel<1, ES, true, false, kCtasPerSmM1b>
+                                    : linear_ccw_kernel<1, ES, true>;
     } else if (kind == 1 && p.probe_ns != 0) {
       if constexpr (ES == 2)
-        kern = p.cluster > 1 ? linear_ccw_kernel<M, ES, true, true> : linear_ccw_kernel<M, ES, false, true>;
+        kern = p.cluster > 1 ? linear_ccw_kernel<1, ES, true, true> : linear_ccw_kernel<1, ES, false, true>;
       else
         return SP_ERR_UNSUPPORTED;
-    } else if (kind == 1)
-      kern = p.cluster > 1 ? linear_ccw_kernel<M, ES, true> : linear_ccw_kernel<M, ES, false>;
-    else
-      kern = p.cluster > 1 ? linear_cc_kernel<M, ES, true> : linear_cc_kernel<M, ES, false>;
+    } else if (kind == 1) {
+      kern = linear_ccw_kernel<1, ES, false>;
+    } else {
+      kern = p.cluster > 1 ? linear_cc_kernel<1, ES, true> : linear_cc_kernel<1, ES, false>;
+    }
   } else {
-    kern = p.cluster > 1 ? linear_cc_kernel<M, ES, true> : linear_cc_kernel<M, ES, false>;
+    // more rows than two: stream-K only
+    if (occ != kCtasPerSm || (p.cluster > 1 && M > 2)) return SP_ERR_UNSUPPORTED;
+    kern = linear_cc_kernel<M, ES, false>;
+    if constexpr (M == 2) {
+      if (p.cluster > 1) kern = linear_cc_kernel<M, ES, true>;
+    }
+    if constexpr (M <= 4) {
+      if (kind == 1 && p.probe_ns != 0) {
+        if constexpr (ES == 2) {
+          kern = linear_ccw_kernel<M, ES, false, true>;
+          if constexpr (M == 2) {
+            if (p.cluster > 1) kern = linear_ccw_kernel<M, ES, true, true>;
+          }
+        } else {
+          return SP_ERR_UNSUPPORTED;
+        }
+      } else if (kind == 1) {
+        kern = linear_ccw_kernel<M, ES, false>;
+        if constexpr (M == 2) {
+          if (p.cluster > 1) kern = linear_ccw_kernel<M, ES, true>;
+        }
+      }
+    }
   }
   static bool configured[5][2][kMaxDevices] = {};  // kernel attributes, once per device
   int dev = 0;
@@ -863,7 +886,7 @@ bool cc_plan(const sp_matrix* h, int Mt, int S, int occ, CcPlan* pl) {
 
 // The launch configuration of one launch with Mt batch rows: six CTAs per SM for a
 // warp-per-chunk cluster launch at M = 1 where its plan fits, else five where that fits,
-// else four; S = 1 (stream-K) without clusters.
+// else four; S = 1 (stream-K) without clusters and for more than two rows.
 bool select_cc(const sp_matrix* h, int Mt, bool allow_cluster, bool probe, int* S, CcPlan* pl) {
   if (allow_cluster && Mt == 1 && !probe) {
     for (const int occ : {kCtasPerSmM1, kCtasPerSmM1b}) {
@@ -874,7 +897,7 @@ bool select_cc(const sp_matrix* h, int Mt, bool allow_cluster, bool probe, int* 
       }
     }
   }
-  *S = allow_cluster ? cluster_cc(h, kCtasPerSm) : 1;
+  *S = allow_cluster && Mt <= 2 ? cluster_cc(h, kCtasPerSm) : 1;
   return cc_plan(h, Mt, *S, kCtasPerSm, pl);
 }
 
@@ -897,10 +920,14 @@ sp_status launch_linear_cc(const sp_matrix* h, const uint16_t* x, int64_t M, uin
   // the configuration depends on the batch rows of a launch: full launches of kMaxTokens
   // rows and one ragged tail; the workspace is checked before the first launch
   const bool probe = probe_ns != 0;
+  // Most batches of more than one row run on linear_mma_kernel, which needs no workspace, except
+  // where the caller wants this file's kernels: the no-allocation entry point and the
+  // failure-path test.
+  auto on_mma = [&](int Mt) { return allow_cluster && !probe && uses_mma(h, Mt); };
   auto stream_k = [&](int Mt) {
     CcPlan q;
     int S = 1;
-    return !select_cc(h, Mt, allow_cluster, probe, &S, &q) || S == 1;
+    return !on_mma(Mt) && (!select_cc(h, Mt, allow_cluster, probe, &S, &q) || S == 1);
   };
   const int tail = (int)(M % kMaxTokens);
   const bool needs_ws = (M >= kMaxTokens && stream_k(kMaxTokens)) || (tail != 0 && stream_k(tail));
@@ -926,6 +953,11 @@ sp_status launch_linear_cc(const sp_matrix* h, const uint16_t* x, int64_t M, uin
   p.chunk_region = (uint32_t)((h->max_chunk + 127) / 128 * 128);
   for (int64_t m0 = 0; m0 < M; m0 += kMaxTokens) {
     const int Mt = (int)std::min<int64_t>(kMaxTokens, M - m0);
+    if (on_mma(Mt)) {
+      const sp_status st = launch_linear_mma(h, x + m0 * h->K, Mt, y + m0 * ldy, stream, epi, r);
+      if (st != SP_OK) return st;
+      continue;
+    }
     int S = 1;
     CcPlan pl;
     if (!select_cc(h, Mt, allow_cluster, probe, &S, &pl)) return SP_ERR_UNSUPPORTED;
@@ -942,7 +974,7 @@ sp_status launch_linear_cc(const sp_matrix* h, const uint16_t* x, int64_t M, uin
     const size_t smem = pl.smem;
     // after an in-place weight update the first launch waits for the whole previous grid
     // (no weight copy may start before its writes are visible)
-    const bool pdl = !(m0 == 0 && h->weights_written);
+    const bool pdl = !h->weights_written;
     const sp_status st = h->esize == 2 ? dispatch_m<2>(p, stream, smem, kind, pl.occ, pdl)
                                         : dispatch_m<1>(p, stream, smem, kind, pl.occ, pdl);
     if (st != SP_OK) return st;

@@ -1,0 +1,600 @@
+// sp_linear_mma.cu -- sparse linear for batches of 2 .. 32 rows: chunks expanded in
+// registers straight into the operands of warp-level matrix instructions.
+//
+// Between one row (linear_ccw_kernel walks the kept weights only) and a few dozen rows the
+// product is bound by neither HBM nor the tensor pipe but by the work of turning a chunk's
+// mask and packed values into operands.  A walk over kept weights on the CUDA cores pays M
+// multiply-adds and M / 2 shuffles per weight; the tcgen05 kernel pays ~250 ns per chunk on
+// its issuing thread (a tcgen05.mma costs ~80 cycles to issue however few tokens it has)
+// plus the trip through tensor memory.  Here a warp expands 16 columns of two rows per lane
+// directly into the A registers of mma.sync m16n8k16 (bf16, FP32 accumulation), so the cost
+// of a chunk hardly depends on M: four matrix instructions per 16 rows and 8 tokens beside
+// ~290 instructions of expansion.  What bounds it is shared memory: ~530 wavefronts per chunk
+// (predicated two-byte value loads at 1.6 each), 62 % of the peak rate over a gate/up launch
+// (ncu), the rest being launch latency and tail.  Measured at 70 %, bf16, graphs of launches on
+// matrices beyond L2, before / here: gate/up 32.2 / 28.1 us at M = 3, 48.7 / 28.4 at M = 5,
+// 61.6 / 31.5 at M = 10, 46.4 / 32.1 at M = 16, 47.2 / 40.9 at M = 32; o 15.3 / 8.8, 18.2 / 9.6,
+// 20.9 / 9.8, 23.4 / 12.8 at M = 5, 10, 16, 32; INT8 gate/up 54 / 34.6 at M = 5, 55.5 / 40.0 at
+// M = 16.
+//
+// The product is free to permute K: in k-step s, lane (g, t) of a warp (g = lane / 4,
+// t = lane % 4) supplies columns 16t + 4s .. 16t + 4s + 3 of its two rows, and of token g of
+// x, so its 16 columns are one contiguous run of a row's values and of x's 128-byte tile row.
+//
+// CTA: one row block's share of K-tiles (a thread-block cluster of S CTAs covers the row
+// block, as in linear_ccw_kernel).
+//   warp CW, lane 0  producer: one cp.async.bulk per chunk and one TMA box of x (8 NT tokens
+//                    x 64 columns, 128-byte swizzle; tokens past M and columns past K read as
+//                    zero) into a ring of `slots` slots, full/empty mbarriers.
+//   warps 0..CW-1    consumers.  128 / RW warps share a chunk, each taking RW of its rows; the
+//                    CTA has CW * RW / 128 chunks in work.  A warp scans the popcounts of its 16-column mask pieces into a table
+//                    (mask piece, first value) of its own, and expands and multiplies 16 rows
+//                    at a time.
+// At the end of its K-tiles a CTA adds its warps' sums in warp order in shared memory (on the
+// ring, which is idle by then); the cluster's CTAs then each sum a share of the tokens over
+// all ranks in rank order (distributed shared memory) and write y through the launch's output
+// epilogue.  All orders are fixed: results are bitwise repeatable.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+
+#include "../../include/sp_stack.h"
+#include "sp_expand.cuh"
+
+namespace sp {
+namespace {
+
+constexpr int kMaxDevices = 64;
+constexpr int kMaxSlots = 16;
+
+struct MmaParams {
+  const uint8_t* buf;
+  const uint64_t* off;
+  const uint64_t* qidx;
+  const float* scale;  // INT8 only
+  uint16_t* y;
+  const uint16_t* r;   // SP_EPI_RESIDUAL
+  int* status;
+  int64_t N, C;        // output rows; chunks
+  int32_t T, M;
+  int32_t cluster;     // CTAs per row block
+  int32_t slots;
+  uint32_t chunk_region, ring_off, tab_off, bar_off;
+  int32_t epi;
+  int32_t early;       // release the next launch as soon as this one's inputs are ready
+  uint64_t timeout_ns;
+};
+
+// volatile: keeps its place among the (volatile) expansion steps, so that the table entries
+// are not all loaded, and held in registers, at once
+__device__ __forceinline__ uint32_t lds32(uint32_t saddr) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(saddr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                         uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, "
+      "%2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// Two columns as bf16x2 from a row's value stream (columns 2P, 2P + 1 of the mask piece m).
+template <int ES, int P>
+__device__ __forceinline__ uint32_t expand2(uint32_t m, uint32_t& pa) {
+  if constexpr (ES == 2)
+    return expand_word_bf16<1u << (2 * P), 2u << (2 * P)>(m, pa);
+  else
+    return i8x2_to_bf16x2(expand_word_u8<1u << (2 * P), 2u << (2 * P)>(m, pa));
+}
+
+// 16 rows (two per lane) x 64 columns against NT token tiles.
+template <int ES, int NT, int S>
+__device__ __forceinline__ void tile_mma(uint32_t m0, uint32_t& pa0, uint32_t m1, uint32_t& pa1,
+                                         const uint32_t (&xb)[NT][8], float (&acc)[NT][4]) {
+  const uint32_t a0 = expand2<ES, 2 * S>(m0, pa0);
+  const uint32_t a1 = expand2<ES, 2 * S>(m1, pa1);
+  const uint32_t a2 = expand2<ES, 2 * S + 1>(m0, pa0);
+  const uint32_t a3 = expand2<ES, 2 * S + 1>(m1, pa1);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[nt], a0, a1, a2, a3, xb[nt][2 * S], xb[nt][2 * S + 1]);
+  if constexpr (S + 1 < 4) tile_mma<ES, NT, S + 1>(m0, pa0, m1, pa1, xb, acc);
+}
+
+// y[m, n] from its FP32 sum v (INT8: times the row's scale sc) through the launch's epilogue
+// (sp_chain_epilogue).  All lanes of a warp call it together with consecutive rows n and one
+// token m; rows past N write nothing.
+__device__ __forceinline__ void write_one(const MmaParams& p, int64_t n, int m, float v, float sc) {
+  const bool in = n < p.N;
+  const uint32_t b = in ? float_to_bf16_bits_rn(v * sc) : 0u;
+  if (p.epi == SP_EPI_PAIR_PRODUCT) {
+    const uint32_t u = __shfl_xor_sync(0xffffffffu, b, 1);
+    if (in && (n & 1) == 0)
+      p.y[(int64_t)m * (p.N >> 1) + (n >> 1)] = float_to_bf16_bits_rn(bf16_bits_to_float(b) * bf16_bits_to_float(u));
+  } else if (in) {
+    uint16_t* yp = p.y + (int64_t)m * p.N + n;
+    if (p.epi == SP_EPI_RESIDUAL)
+      *yp = float_to_bf16_bits_rn(
+          (bf16_bits_to_float(__ldcg(reinterpret_cast<const unsigned short*>(yp))) + bf16_bits_to_float(b)) +
+          bf16_bits_to_float(p.r[n]));
+    else
+      *yp = (uint16_t)b;
+  }
+}
+
+template <int NT, int ES, int RW, int CW, int OCC>
+__global__ void __launch_bounds__((CW + 1) * 32, OCC)
+    linear_mma_kernel(const __grid_constant__ MmaParams p, const __grid_constant__ CUtensorMap tmap_x) {
+  extern __shared__ __align__(1024) uint8_t smem[];
+  constexpr int kParts = kRows / RW;       // warps that share a chunk
+  constexpr int kGroups = CW / kParts;     // chunks in work at once
+  constexpr int R = RW / 32;               // rows per lane in the scan
+  constexpr int kTiles = RW / 16;          // 16-row tiles of a warp
+  constexpr uint32_t kXBytes = NT * 1024u;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int slots = p.slots;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.bar_off);
+  uint64_t* empty = full + kMaxSlots;
+  uint64_t* qx = empty + kMaxSlots;                                   // quarter index of each slot's chunk
+  volatile int* tag = reinterpret_cast<volatile int*>(qx + kMaxSlots);  // item each slot was claimed for
+  const int T = p.T;
+  const int64_t seg = blockIdx.x / p.cluster;  // row block
+  const int rank = blockIdx.x % p.cluster;
+  const int t0 = (int)((int64_t)rank * T / p.cluster), t1 = (int)((int64_t)(rank + 1) * T / p.cluster);
+  const int n_items = t1 - t0;
+
+  if (tid == 0) {
+    for (int s = 0; s < slots; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], kParts);
+      tag[s] = -1;
+    }
+    fence_barrier_init();
+  }
+  __syncthreads();
+
+  if (warp == CW) {
+    // ------------------------------------------------------------ producer
+    const uint64_t pol = policy_evict_first();
+    const int64_t c0 = seg * T + t0;
+    int64_t base = -64;  // offsets (and quarter indices) of chunks base .. base + 31, one per lane
+    uint64_t vo = 0, vq = 0;
+    auto chunk_at = [&](int i, uint64_t* o0, uint64_t* o1, uint64_t* qi) {
+      const int64_t c = c0 + i;
+      if (c - base >= 31 || c < base) {
+        base = c;
+        vo = c + lane <= p.C ? __ldg(p.off + c + lane) : 0ull;
+        if (kParts > 1) vq = c + lane < p.C ? __ldg(p.qidx + c + lane) : 0ull;
+      }
+      *o0 = __shfl_sync(0xffffffffu, vo, (int)(c - base));
+      *o1 = __shfl_sync(0xffffffffu, vo, (int)(c - base) + 1);
+      if (kParts > 1) *qi = __shfl_sync(0xffffffffu, vq, (int)(c - base));
+    };
+    auto issue_chunk = [&](int i, int s, uint64_t o0, uint64_t o1, uint64_t qi) {
+      const uint32_t bytes = (uint32_t)(o1 - o0);
+      if (kGroups > 1) tag[s] = i;
+      if (kParts > 1) qx[s] = qi;
+      mbar_arrive_expect_tx(&full[s], bytes + kXBytes);
+      bulk_g2s_hint(smem + p.ring_off + (size_t)s * p.chunk_region, p.buf + o0, bytes, &full[s], pol);
+    };
+    if (lane == 0) prefetch_tmap(&tmap_x);
+    const int n_pre = n_items < slots ? n_items : slots;
+    for (int i = 0; i < n_pre; ++i) {  // weight bytes do not depend on the previous grid
+      uint64_t o0, o1, qi = 0;
+      chunk_at(i, &o0, &o1, &qi);
+      if (lane == 0) issue_chunk(i, i, o0, o1, qi);
+    }
+    pdl_wait();
+    if (p.early) pdl_launch_dependents();
+    int s = 0;
+    uint32_t ph = 0;
+    bool failed = false;
+    for (int i = 0; i < n_items; ++i) {
+      if (i >= n_pre) {
+        uint64_t o0, o1, qi = 0;
+        chunk_at(i, &o0, &o1, &qi);
+        if (lane == 0) {
+          if (!mbar_wait(&empty[s], ph ^ 1u, p.timeout_ns)) {
+            set_status(p.status, kStatusTimeout);
+            failed = true;
+          } else {
+            issue_chunk(i, s, o0, o1, qi);
+          }
+        }
+        failed = __shfl_sync(0xffffffffu, failed, 0);
+        if (failed) break;
+      }
+      if (lane == 0) tma_load_2d(smem + (size_t)s * kXBytes, &tmap_x, kTileK * (t0 + i), 0, &full[s]);
+      if (++s == slots) {
+        s = 0;
+        ph ^= 1u;
+      }
+    }
+    return;
+  }
+
+  // -------------------------------------------------------------- consumers
+  pdl_wait();
+  if (p.early) pdl_launch_dependents();
+  const int grp = warp / kParts, part = warp % kParts;
+  const int g = lane >> 2, t = lane & 3;
+  // The table entry of piece t of row 8q + g of the warp's rows is word 4 * (8q + (g ^ (q % R))) + t:
+  // a tile's loads are one 128-byte line, and the turn by q keeps the 16-byte stores of the scan,
+  // in which lane l writes rows R l .. R l + R - 1, off each other's banks.
+  uint32_t* tab = reinterpret_cast<uint32_t*>(smem + p.tab_off) + warp * RW * 4;
+  const uint32_t tab_lane = smem_u32(tab) + 16u * g + 4u * t;
+  const int turn = R == 4 ? (lane >> 1) & 3 : R == 2 ? (lane >> 2) & 1 : 0;
+  float acc[kTiles][NT][4];
+#pragma unroll
+  for (int i = 0; i < kTiles; ++i)
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[i][nt][c] = 0.f;
+  bool dead = false;
+  int s = grp;
+  uint32_t ph = 0;
+  for (int n = grp; n < n_items; n += kGroups) {
+    if (kGroups > 1 && !dead && tag[s] != n) {
+      // the slot may still hold an earlier item of another warp: wait until the producer has
+      // claimed it for this one, so that the parity wait below cannot match an older phase
+      const uint64_t w0 = global_ns();
+      while (tag[s] != n) {
+        __nanosleep(32);
+        if (global_ns() - w0 > p.timeout_ns) {
+          dead = true;
+          set_status(p.status, kStatusTimeout);
+          break;
+        }
+      }
+      dead = __any_sync(0xffffffffu, dead);
+    }
+    if (!dead && !__all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.timeout_ns))) {
+      dead = true;
+      set_status(p.status, kStatusTimeout);
+    }
+    if (!dead) {
+      const uint8_t* chunk = smem + p.ring_off + (size_t)s * p.chunk_region;
+      // ---- table: lane l scans rows R l .. R l + R - 1 of the warp's part
+      {
+        uint32_t w[2 * R];  // mask words, 32 columns each
+        if constexpr (R == 1) {
+          const uint2 a = reinterpret_cast<const uint2*>(chunk)[part * RW + lane];
+          w[0] = a.x, w[1] = a.y;
+        } else {
+#pragma unroll
+          for (int i = 0; i < R / 2; ++i) {
+            const uint4 a = reinterpret_cast<const uint4*>(chunk)[part * (RW / 2) + lane * (R / 2) + i];
+            w[4 * i] = a.x, w[4 * i + 1] = a.y, w[4 * i + 2] = a.z, w[4 * i + 3] = a.w;
+          }
+        }
+        int before[4 * R], run = 0;
+#pragma unroll
+        for (int i = 0; i < 2 * R; ++i) {
+          before[2 * i] = run;
+          before[2 * i + 1] = run + __popc(w[i] & 0xffffu);
+          run += __popc(w[i]);
+        }
+        int incl = run;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int u = __shfl_up_sync(0xffffffffu, incl, d);
+          if (lane >= d) incl += u;
+        }
+        int e0 = incl - run;
+        if constexpr (kParts > 1) {  // kept entries before rows 32, 64, 96: the chunk's quarter index
+          const uint64_t qi = qx[s];
+          if (part > 0) e0 += (int)((qi >> (16 * (part * (RW / 32) - 1))) & 0xffffu);
+        }
+        __syncwarp();  // the last chunk's reads of the table
+#pragma unroll
+        for (int e = 0; e < R; ++e) {
+          uint32_t v[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            v[k] = __byte_perm(w[2 * e + (k >> 1)], (uint32_t)(e0 + before[4 * e + k]), (k & 1) ? 0x5432 : 0x5410);
+          reinterpret_cast<uint4*>(tab)[R * lane + (e ^ turn)] = make_uint4(v[0], v[1], v[2], v[3]);
+        }
+        __syncwarp();
+      }
+      // ---- x: token 8 nt + g, columns 16t .. 16t + 15 (two 16-byte pieces of its swizzled row)
+      uint32_t xb[NT][8];
+      const uint8_t* xs = smem + (size_t)s * kXBytes + g * 128;
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        const uint4 a = *reinterpret_cast<const uint4*>(xs + nt * 1024 + (((2 * t) ^ g) << 4));
+        const uint4 b = *reinterpret_cast<const uint4*>(xs + nt * 1024 + (((2 * t + 1) ^ g) << 4));
+        xb[nt][0] = a.x, xb[nt][1] = a.y, xb[nt][2] = a.z, xb[nt][3] = a.w;
+        xb[nt][4] = b.x, xb[nt][5] = b.y, xb[nt][6] = b.z, xb[nt][7] = b.w;
+      }
+      const uint32_t vbase = smem_u32(chunk) + kMaskBytes;
+#pragma unroll
+      for (int i = 0; i < kTiles; ++i) {
+        // rows 16 i + g and 16 i + 8 + g of the warp's part
+        const uint32_t en0 = lds32((tab_lane ^ (16u * ((2 * i) % R))) + 256u * i);
+        const uint32_t en1 = lds32((tab_lane ^ (16u * ((2 * i + 1) % R))) + 256u * i + 128u);
+        uint32_t pa0 = vbase + (en0 >> 16) * ES, pa1 = vbase + (en1 >> 16) * ES;
+        tile_mma<ES, NT, 0>(en0, pa0, en1, pa1, xb, acc[i]);
+      }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s]);
+    if ((s += kGroups) >= slots) {
+      s -= slots;
+      ph ^= 1u;
+    }
+  }
+
+  // ---------------------------------------------------------------- the CTA's sums
+  // Every copy into the ring has landed (its item was waited for), so the ring's memory now
+  // holds the partials: [kGroups][M][kRows] floats, group 0's part becoming the CTA's sum.
+  named_bar_sync(1, CW * 32);
+  const int M = p.M;
+  float* comb = reinterpret_cast<float*>(smem);
+#pragma unroll
+  for (int i = 0; i < kTiles; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int row = part * RW + 16 * i + 8 * (c >> 1) + g;
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        const int tok = 8 * nt + 2 * t + (c & 1);
+        if (tok < M) comb[(grp * M + tok) * kRows + row] = acc[i][nt][c];
+      }
+    }
+  named_bar_sync(1, CW * 32);
+  // warps 4h .. 4h + 3 take tokens h, h + CW / 4, ...; a thread takes one row
+  constexpr int kStep = CW / 4;
+  const int rr = tid % kRows, m0 = tid / kRows;
+  const int64_t row = seg * kRows + rr;
+  const float sc = (ES == 1 && row < p.N) ? p.scale[row] : 1.f;
+  if (p.cluster == 1) {
+    for (int m = m0; m < M; m += kStep) {
+      float v = comb[m * kRows + rr];
+#pragma unroll
+      for (int q = 1; q < kGroups; ++q) v += comb[(q * M + m) * kRows + rr];
+      write_one(p, row, m, v, sc);
+    }
+    return;
+  }
+  if constexpr (kGroups > 1) {
+    for (int m = m0; m < M; m += kStep) {
+      float v = comb[m * kRows + rr];
+#pragma unroll
+      for (int q = 1; q < kGroups; ++q) v += comb[(q * M + m) * kRows + rr];
+      comb[m * kRows + rr] = v;
+    }
+  }
+  cluster_sync_all();
+  const uint32_t mine = smem_u32(comb) + 4u * (uint32_t)rr;
+  for (int m = rank + m0 * p.cluster; m < M; m += kStep * p.cluster) {
+    float v = 0.f;
+#pragma unroll 4
+    for (int q = 0; q < p.cluster; ++q) v += ld_cluster_f32(cluster_map(mine + 4u * (uint32_t)(m * kRows), (uint32_t)q));
+    write_one(p, row, m, v, sc);
+  }
+  cluster_sync_all();  // every CTA's sums stay until the others have read them
+}
+
+// ------------------------------------------------------------------ host side
+// Token tiles, rows per warp, consumer warps, CTAs per SM (at most) and per row block.
+struct MmaChoice {
+  int nt, rw, cw, occ, cluster;
+};
+struct MmaPlan {
+  int slots, cluster;
+  uint32_t chunk_region, ring_off, tab_off, bar_off;
+  size_t smem;
+};
+
+// Largest cluster size of 2 .. 8 and 16 (9 .. 15 place badly) that keeps rb * S within `cap` CTAs
+// and leaves a CTA at least `cmin` of the T K-tiles; 1 (a CTA per row block) otherwise.
+int cluster_size(int64_t rb, int64_t T, int64_t cap, int cmin) {
+  for (int64_t S = std::min<int64_t>(16, cap / rb); S > 1; --S)
+    if ((S <= 8 || S == 16) && T / S >= cmin) return (int)S;
+  return 1;
+}
+
+// A grid overlaps well with the launches around it if it fills the CTA slots to 80 % (the next
+// grid's CTAs then follow its exits evenly) or leaves half of them free (the next grid fits
+// beside it whole).  In between, part of the next grid gets in and the rest waits for the
+// tail: such a grid keeps the next launch out until it exits.  Measured at M = 4, 70 %, next
+// launch released early / at exit: 256 CTAs of 912 slots 8.5 / 10.3 us (o), 860 of 912
+// 28.6 / 29.2 us (gate/up), but 512 of 912 22.1 / 18.3 us (down).
+bool fills(int64_t grid, int64_t slots) { return grid * 5 >= slots * 4; }
+bool overlaps(int64_t grid, int64_t slots) { return grid * 2 <= slots || fills(grid, slots); }
+
+// More than 20 chunks per SM: throughput counts, below mostly latency.
+bool large(const sp_matrix* h) { return (int64_t)h->RB * h->T > 20 * (int64_t)h->num_sms; }
+
+// The launch of a batch of M <= kMmaMaxRows rows.  Two forms per token count: four consumer
+// warps at a high occupancy, and eight, whose share of a row block per warp is shorter.
+//  * Small matrices: best is one eight-warp CTA per SM
+//    with as large a cluster as that allows, which also leaves room for the whole next grid:
+//    o (32 row blocks) 8.4 -> 7.8 us at M = 2 against 256 four-warp CTAs, 8192 x 2048 8.4 -> 7.9.
+//    With more row blocks than SMs, four warps and the largest cluster whose grid overlaps:
+//    22016 x 512 8.3 -> 6.1 us against a CTA per row block released at exit.
+//  * Larger matrices want every CTA slot full: eight warps where their grid fills the slots,
+//    else four.  q/k/v (96 row blocks) 17.8 us with eight, 18.5 with four at M = 4, 20.3 / 21.5
+//    at M = 16; down (32) 16.5 / 17.2 at M = 2 (80 %), 19.5 / 20.9 at M = 16; gate/up (172, eight
+//    warps leave a quarter of the slots empty) 30.8 / 28.6 at M = 4, 41.0 / 32.4 at M = 16.
+MmaChoice choose(const sp_matrix* h, int M) {
+  const int nt = M <= 8 ? 1 : M <= 16 ? 2 : 4;
+  const MmaChoice few = nt == 1 ? MmaChoice{1, 64, 4, 6, 1} : nt == 2 ? MmaChoice{2, 32, 4, 5, 1} : MmaChoice{4, 32, 4, 4, 1};
+  const MmaChoice many = nt == 1 ? MmaChoice{1, 64, 8, 3, 1} : nt == 2 ? MmaChoice{2, 64, 8, 2, 1} : MmaChoice{4, 32, 8, 2, 1};
+  const int64_t rb = std::max<int32_t>(h->RB, 1), T = h->T, sms = h->num_sms;
+  MmaChoice c = few;
+  if (!large(h)) {
+    if (rb <= sms) {
+      c = many;
+      c.occ = 2;
+      c.cluster = cluster_size(rb, T, sms, 2);
+      return c;
+    }
+    const int64_t slots = c.occ * sms;
+    for (int64_t S = std::min<int64_t>(8, slots / rb); S > 1; --S)
+      if (T / S >= 2 && overlaps(rb * S, slots)) {
+        c.cluster = (int)S;
+        break;
+      }
+    return c;
+  }
+  for (int occ = many.occ; occ >= 2; --occ) {
+    const int S = cluster_size(rb, T, occ * sms, 8);
+    if (fills(rb * S, occ * sms) && rb * S <= occ * sms) {
+      c = many;
+      c.occ = occ;
+      c.cluster = S;
+      return c;
+    }
+  }
+  c.cluster = cluster_size(rb, T, c.occ * sms, 8);
+  return c;
+}
+
+// Ring slots and shared-memory layout for `occ` CTAs per SM; false if fewer than `min_slots` fit.
+bool mma_plan(const sp_matrix* h, int M, const MmaChoice& c, int occ, int min_slots, MmaPlan* pl) {
+  pl->cluster = c.cluster;
+  pl->chunk_region = (uint32_t)((h->max_chunk + 127) / 128 * 128);
+  const size_t budget = (size_t)(227 * 1024) / occ - 1024;
+  const size_t tab = (size_t)c.cw * c.rw * 16;
+  const size_t ctl = (size_t)kMaxSlots * (8 + 8 + 8 + 4);
+  const size_t per_slot = (size_t)c.nt * 1024 + pl->chunk_region;
+  if (budget < tab + ctl + min_slots * per_slot) return false;
+  const int items = (h->T + pl->cluster - 1) / pl->cluster;
+  pl->slots = (int)std::min<size_t>(std::min<size_t>(kMaxSlots, std::max(items, min_slots)),
+                                    (budget - tab - ctl) / per_slot);
+  pl->ring_off = (uint32_t)(pl->slots * c.nt * 1024);
+  const size_t sums = (size_t)(c.cw * c.rw / kRows) * M * kRows * sizeof(float);  // on the ring
+  const size_t ring_end = std::max<size_t>(pl->ring_off + (size_t)pl->slots * pl->chunk_region, (sums + 127) / 128 * 128);
+  pl->tab_off = (uint32_t)ring_end;
+  pl->bar_off = (uint32_t)(ring_end + tab);
+  // The whole share of shared memory, whatever the chunks need: CTAs of consecutive launches
+  // then fit the holes that each other's leave.  Sizes following the largest chunk cost 33.2
+  // instead of 27.9 us (gate/up, M = 4) between matrices 128 bytes apart, because the larger
+  // CTA does not fit where the smaller one was.
+  pl->smem = budget / 128 * 128;
+  return true;
+}
+
+template <int NT, int ES, int RW, int CW, int OCC>
+sp_status launch(const sp_matrix* h, const MmaParams& p, const CUtensorMap& map, const MmaPlan& pl,
+                 cudaStream_t stream, bool pdl) {
+  auto kern = linear_mma_kernel<NT, ES, RW, CW, OCC>;
+  static bool configured[kMaxDevices] = {};
+  const int dev = h->device;
+  if (dev < 0 || dev >= kMaxDevices) return SP_ERR_UNSUPPORTED;
+  if (!configured[dev]) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      cudaGetLastError();
+      return SP_ERR_CUDA;
+    }
+    configured[dev] = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(h->RB * pl.cluster));
+  cfg.blockDim = dim3((CW + 1) * 32);
+  cfg.dynamicSmemBytes = pl.smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)pl.cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pl.cluster > 1 ? 2 : 1;
+  if (cudaLaunchKernelEx(&cfg, kern, p, map) != cudaSuccess) {
+    cudaGetLastError();
+    return SP_ERR_CUDA;
+  }
+  return SP_OK;
+}
+
+// The plan for `c`, at the largest occupancy up to c.occ whose ring holds a slot per chunk in
+// work and one more (a dense matrix's chunks are ~17 KB).
+bool plan_for(const sp_matrix* h, int M, const MmaChoice& c, MmaPlan* pl) {
+  const int groups = c.cw * c.rw / kRows;
+  for (int occ = c.occ; occ >= 1; --occ)
+    if (mma_plan(h, M, c, occ, groups < 4 ? groups + 1 : groups, pl)) return true;
+  return false;
+}
+
+template <int ES>
+sp_status dispatch(const sp_matrix* h, const MmaParams& p, const CUtensorMap& map, const MmaPlan& pl,
+                   const MmaChoice& c, cudaStream_t stream, bool pdl) {
+  if (c.nt == 1)
+    return c.cw == 4 ? launch<1, ES, 64, 4, 6>(h, p, map, pl, stream, pdl)
+                     : launch<1, ES, 64, 8, 3>(h, p, map, pl, stream, pdl);
+  if (c.nt == 2)
+    return c.cw == 4 ? launch<2, ES, 32, 4, 5>(h, p, map, pl, stream, pdl)
+                     : launch<2, ES, 64, 8, 2>(h, p, map, pl, stream, pdl);
+  return c.cw == 4 ? launch<4, ES, 32, 4, 4>(h, p, map, pl, stream, pdl)
+                   : launch<4, ES, 32, 8, 2>(h, p, map, pl, stream, pdl);
+}
+
+}  // namespace
+
+// Two rows of a large matrix stay with the kept-weight walk (M = 2, 80 %: down 15.0 us against
+// 17.1 here; INT8 at 70 % 20.2 / 21.9; the other shapes within a few percent of each other).
+bool uses_mma(const sp_matrix* h, int64_t M) {
+  if (M < 2 || M > kMmaMaxRows || (M == 2 && large(h))) return false;
+  MmaPlan pl;
+  return plan_for(h, (int)M, choose(h, (int)M), &pl);
+}
+
+sp_status launch_linear_mma(const sp_matrix* h, const uint16_t* x, int64_t M, uint16_t* y, cudaStream_t stream,
+                            int32_t epi, const uint16_t* r) {
+  if (M < 1 || M > kMmaMaxRows) return SP_ERR_UNSUPPORTED;
+  const MmaChoice c = choose(h, (int)M);
+  MmaPlan pl;
+  if (!plan_for(h, (int)M, c, &pl)) return SP_ERR_UNSUPPORTED;
+  PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  sp_status st = tensor_map_encoder(&encode);
+  if (st != SP_OK) return st;
+  MmaParams p{};
+  p.buf = h->d_buf;
+  p.off = h->d_off;
+  p.qidx = h->d_qidx;
+  p.scale = h->d_scale;
+  p.y = y;
+  p.r = r;
+  p.status = device_status_ptr();
+  p.N = h->N;
+  p.C = (int64_t)h->RB * h->T;
+  p.T = h->T;
+  p.M = (int32_t)M;
+  p.cluster = pl.cluster;
+  p.slots = pl.slots;
+  p.chunk_region = pl.chunk_region;
+  p.ring_off = pl.ring_off;
+  p.tab_off = pl.tab_off;
+  p.bar_off = pl.bar_off;
+  p.epi = epi;
+  p.early = overlaps((int64_t)h->RB * pl.cluster, (int64_t)c.occ * h->num_sms) ? 1 : 0;
+  p.timeout_ns = wait_timeout_ns();
+  // x [M, K] bf16, box = 64 columns x 8 NT tokens, 128-byte swizzle; rows past M and columns
+  // past K read as zero
+  CUtensorMap map;
+  const cuuint64_t gdim[2] = {(cuuint64_t)h->K, (cuuint64_t)M};
+  const cuuint64_t gstride[1] = {(cuuint64_t)h->K * 2};
+  const cuuint32_t box[2] = {(cuuint32_t)kTileK, (cuuint32_t)(8 * c.nt)};
+  const cuuint32_t estride[2] = {1, 1};
+  if (encode(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(x), gdim, gstride, box, estride,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return SP_ERR_CUDA;
+  // after an in-place weight update the launch waits for the whole previous grid (no weight
+  // copy may start before its writes are visible)
+  const bool pdl = !h->weights_written;
+  st = h->esize == 2 ? dispatch<2>(h, p, map, pl, c, stream, pdl) : dispatch<1>(h, p, map, pl, c, stream, pdl);
+  if (st == SP_OK) h->weights_written = 0;
+  return st;
+}
+
+}  // namespace sp

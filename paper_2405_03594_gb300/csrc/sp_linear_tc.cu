@@ -663,6 +663,7 @@ size_t workspace_bytes_tc(const sp_matrix* h, int64_t M) {
 sp_status launch_linear_tc(const sp_matrix* h, const uint16_t* x, int64_t M, uint16_t* y, void* ws, size_t ws_bytes,
                            cudaStream_t stream) {
   if (!ws || ws_bytes < workspace_bytes_tc(h, M)) return SP_ERR_WORKSPACE;
+  if (uses_mma(h, M)) return launch_linear_mma(h, x, M, y, stream, 0, nullptr);
   if (M > ((int64_t)1 << 31) / kMaxNtok) return SP_ERR_UNSUPPORTED;
   PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   sp_status st = tensor_map_encoder(&encode);
