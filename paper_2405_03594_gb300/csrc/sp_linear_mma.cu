@@ -459,7 +459,7 @@ MmaChoice choose(const sp_matrix* h, int M) {
 bool mma_plan(const sp_matrix* h, int M, const MmaChoice& c, int occ, int min_slots, MmaPlan* pl) {
   pl->cluster = c.cluster;
   pl->chunk_region = (uint32_t)((h->max_chunk + 127) / 128 * 128);
-  const size_t budget = (size_t)(227 * 1024) / occ - 1024;
+  const size_t budget = ((size_t)(227 * 1024) / occ - 1024) / 128 * 128;  // all of it is asked for
   const size_t tab = (size_t)c.cw * c.rw * 16;
   const size_t ctl = (size_t)kMaxSlots * (8 + 8 + 8 + 4);
   const size_t per_slot = (size_t)c.nt * 1024 + pl->chunk_region;
@@ -472,11 +472,12 @@ bool mma_plan(const sp_matrix* h, int M, const MmaChoice& c, int occ, int min_sl
   const size_t ring_end = std::max<size_t>(pl->ring_off + (size_t)pl->slots * pl->chunk_region, (sums + 127) / 128 * 128);
   pl->tab_off = (uint32_t)ring_end;
   pl->bar_off = (uint32_t)(ring_end + tab);
+  if (pl->bar_off + ctl > budget) return false;
   // The whole share of shared memory, whatever the chunks need: CTAs of consecutive launches
   // then fit the holes that each other's leave.  Sizes following the largest chunk cost 33.2
   // instead of 27.9 us (gate/up, M = 4) between matrices 128 bytes apart, because the larger
   // CTA does not fit where the smaller one was.
-  pl->smem = budget / 128 * 128;
+  pl->smem = budget;
   return true;
 }
 
