@@ -111,8 +111,9 @@ sp_status sp_compress(const void* w_dev, const uint8_t* mask_dev, int64_t n, int
  * SP_ERR_BAD_HANDLE for a dead handle, SP_ERR_INVALID_ARG for a null output. */
 sp_status sp_decompress(const sp_matrix* h, void* w_out_dev, void* stream);
 
-/* Bytes of device workspace that sp_linear needs for a batch of m rows (its split-K scratch;
- * library plumbing with no counterpart in the paper), written to *bytes (0 for m == 0).  Host only.  SP_ERR_INVALID_ARG for m < 0 or a null `bytes`. */
+/* Bytes of device workspace that sp_linear needs for a batch of m rows (its split-K scratch, or
+ * for large batches room for the expanded matrix, 2 bytes per weight; library plumbing with no
+ * counterpart in the paper), written to *bytes (0 for m == 0).  Host only.  SP_ERR_INVALID_ARG for m < 0 or a null `bytes`. */
 sp_status sp_workspace_size(const sp_matrix* h, int64_t m, size_t* bytes);
 
 /* y = x . (W o Mask)^T, FP32 accumulation, bf16 output (round to nearest even): the sparse
@@ -146,7 +147,8 @@ enum {
 /* (Library plumbing; no counterpart in the paper.)  Number of kernel launches that
  * sp_linear_ex(h, x, m, y, ws, ws_bytes, path, stream)
  * makes, written to *launches: 0 for m == 0, one per 16 batch rows on the CUDA-core
- * family, one on the tensor-core family; if `kernel` is not null, the SP_KERNEL_* value
+ * family, one on the tensor-core family, or two where it expands the matrix first (large
+ * batches); if `kernel` is not null, the SP_KERNEL_* value
  * of the kernel used for the first 16 rows (or all rows) goes there.  For callers that
  * count launches or label profiles.  Host only: no GPU work.  SP_ERR_BAD_HANDLE for a
  * dead handle, SP_ERR_INVALID_ARG for m < 0, an unknown path or a null `launches`. */

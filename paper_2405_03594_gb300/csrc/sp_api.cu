@@ -29,6 +29,12 @@ bool live(const sp_matrix* h) { return h && h->magic == SP_MAGIC; }
 constexpr int64_t kCudaCoreMaxM_bf16 = 10;
 constexpr int64_t kCudaCoreMaxM_int8 = 13;
 
+// Workspace of the documented contract, whatever kernel runs a batch of m rows.
+size_t workspace_bytes(const sp_matrix* h, int64_t m) {
+  const size_t b = std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m));
+  return uses_dense(h, m) ? std::max(b, workspace_bytes_dense(h)) : b;
+}
+
 bool uses_tensor_cores(const sp_matrix* h, int64_t m, sp_path path) {
   const int64_t cc_max = h->esize == 1 ? kCudaCoreMaxM_int8 : kCudaCoreMaxM_bf16;
   return path == SP_PATH_TENSOR_CORE || (path == SP_PATH_AUTO && m > cc_max);
@@ -108,7 +114,7 @@ sp_status sp_decompress(const sp_matrix* h, void* w_out_dev, void* stream) {
 sp_status sp_workspace_size(const sp_matrix* h, int64_t m, size_t* bytes) {
   if (!live(h)) return SP_ERR_BAD_HANDLE;
   if (!bytes || m < 0) return SP_ERR_INVALID_ARG;
-  *bytes = m == 0 ? 0 : std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m));
+  *bytes = m == 0 ? 0 : workspace_bytes(h, m);
   return SP_OK;
 }
 
@@ -126,8 +132,7 @@ sp_status sp_linear_ex(const sp_matrix* h, const void* x_dev, int64_t m, void* y
     return SP_ERR_CUDA;
   }
   if (dev != h->device) return SP_ERR_INVALID_ARG;
-  // The documented contract, whatever kernel runs: a workspace of sp_workspace_size bytes.
-  if (!workspace_dev || workspace_bytes < std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m)))
+  if (!workspace_dev || workspace_bytes < sp::workspace_bytes(h, m))
     return SP_ERR_WORKSPACE;
   if (uses_tensor_cores(h, m, path))
     return launch_linear_tc(h, static_cast<const uint16_t*>(x_dev), m, static_cast<uint16_t*>(y_dev), workspace_dev,
@@ -155,7 +160,7 @@ sp_status sp_linear_epi(const sp_matrix* h, const void* x_dev, int64_t m, void* 
     return SP_ERR_CUDA;
   }
   if (dev != h->device) return SP_ERR_INVALID_ARG;
-  if (!workspace_dev || workspace_bytes < std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m)))
+  if (!workspace_dev || workspace_bytes < sp::workspace_bytes(h, m))
     return SP_ERR_WORKSPACE;
   if (uses_tensor_cores(h, m, SP_PATH_AUTO)) return SP_ERR_UNSUPPORTED;
   return launch_linear_cc(h, static_cast<const uint16_t*>(x_dev), m, static_cast<uint16_t*>(y_dev), workspace_dev,
@@ -168,7 +173,7 @@ sp_status sp_launch_count(const sp_matrix* h, int64_t m, sp_path path, int64_t* 
   if (m < 0 || !launches || (path != SP_PATH_AUTO && path != SP_PATH_CUDA_CORE && path != SP_PATH_TENSOR_CORE))
     return SP_ERR_INVALID_ARG;
   const bool tc = uses_tensor_cores(h, m, path);
-  *launches = m == 0 ? 0 : tc ? 1 : (m + kMaxTokens - 1) / kMaxTokens;
+  *launches = m == 0 ? 0 : tc ? (uses_dense(h, m) ? 2 : 1) : (m + kMaxTokens - 1) / kMaxTokens;
   if (kernel) {
     if (m == 0)
       *kernel = SP_KERNEL_NONE;
@@ -197,7 +202,7 @@ sp_status sp_test_expired_wait(const sp_matrix* h, const void* x_dev, int64_t m,
     return SP_ERR_CUDA;
   }
   if (dev != h->device) return SP_ERR_INVALID_ARG;
-  if (!workspace_dev || workspace_bytes < std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m)))
+  if (!workspace_dev || workspace_bytes < sp::workspace_bytes(h, m))
     return SP_ERR_WORKSPACE;
   return launch_linear_cc(h, static_cast<const uint16_t*>(x_dev), m, static_cast<uint16_t*>(y_dev), workspace_dev,
                           workspace_bytes, (cudaStream_t)stream, true, (uint64_t)wait_ms * 1000000ull);
