@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
       }
     }
   } else if (warp == 1) {
-    if (rank == 0 && lane == 0) {
+    if (rank == 0) {
       // ---------------------------------------------------------- MMA issuer (leader)
       int s = 0;
       uint32_t ph = 0;
@@ -246,31 +246,34 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
         const uint32_t idesc = idesc_bf16(kTileRows, ntok);
         const int db = (int)(k & 1);
         const uint32_t d = tmem + (uint32_t)db * kMaxTok;
-        if (k >= 2 && !mbar_wait_cluster(&d_empty[db], (uint32_t)((k / 2 - 1) & 1), p.timeout_ns)) {
+        if (k >= 2 && !__all_sync(0xffffffffu, mbar_wait(&d_empty[db], (uint32_t)((k / 2 - 1) & 1), p.timeout_ns))) {
           set_status(p.status, kStatusTimeout);
           dead = true;
           break;
         }
         tc_fence_after();
         for (int t = 0; t < T; ++t) {
-          if (!mbar_wait_cluster(&full[s], ph, p.timeout_ns)) {
+          if (!__all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.timeout_ns))) {
             set_status(p.status, kStatusTimeout);
             dead = true;
             break;
           }
           tc_fence_after();
           const uint32_t a = smem_u32(smem + kRingOff + (size_t)s * p.stage_bytes);
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_ss2(d, smem_desc_sw128(a + kk * 32u), smem_desc_sw128(a + kABytes + kk * 32u), idesc,
-                    (t > 0 || kk > 0) ? 1u : 0u);
-          mma_commit2(&empty[s]);
+            for (int kk = 0; kk < 4; ++kk)
+              mma_ss2(d, smem_desc_sw128(a + kk * 32u), smem_desc_sw128(a + kABytes + kk * 32u), idesc,
+                      (t > 0 || kk > 0) ? 1u : 0u);
+            mma_commit2(&empty[s]);
+            if (t == T - 1) mma_commit2(&d_full[db]);
+          }
+          __syncwarp();
           if (++s == p.stages) {
             s = 0;
             ph ^= 1u;
           }
         }
-        if (!dead) mma_commit2(&d_full[db]);
       }
     }
   } else if (warp >= kEpiWarp0) {
@@ -289,7 +292,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
       int ntok;
       tile_at(p, i, &rt, &tok0, &ntok);
       const int db = (int)(k & 1);
-      if (!dead && !__all_sync(0xffffffffu, mbar_wait_cluster(&d_full[db], (uint32_t)((k / 2) & 1), p.timeout_ns))) {
+      if (!dead && !__all_sync(0xffffffffu, mbar_wait(&d_full[db], (uint32_t)((k / 2) & 1), p.timeout_ns))) {
         set_status(p.status, kStatusTimeout);
         dead = true;
       }

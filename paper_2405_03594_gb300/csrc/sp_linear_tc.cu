@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(tc_threads(EG), 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    {
       pdl_wait();
       pdl_launch_dependents();
       const uint32_t idesc = idesc_bf16(kRows, tp.ntok);
@@ -327,17 +327,17 @@ __global__ void __launch_bounds__(tc_threads(EG), 1)
           // D buffer reuse: wait for the (k / n_d - 1)-th completion of d_empty[db], the
           // epilogue of segment k - n_d
           if (!dead && k >= n_d) {
-            if (!mbar_wait(&d_empty[db], (uint32_t)((k / n_d - 1) & 1), p.timeout_ns)) {
+            if (!__all_sync(~0u, mbar_wait(&d_empty[db], (uint32_t)((k / n_d - 1) & 1), p.timeout_ns))) {
               dead = true;
               set_status(p.status, kStatusTimeout);
             }
           }
         }
-        if (!dead && !mbar_wait(&full[s], ph, p.timeout_ns)) {
+        if (!dead && !__all_sync(~0u, mbar_wait(&full[s], ph, p.timeout_ns))) {
           dead = true;
           set_status(p.status, kStatusTimeout);
         }
-        if (!dead && !mbar_wait(&a_full[s], ph, p.timeout_ns)) {
+        if (!dead && !__all_sync(~0u, mbar_wait(&a_full[s], ph, p.timeout_ns))) {
           dead = true;
           set_status(p.status, kStatusTimeout);
         }
@@ -345,13 +345,16 @@ __global__ void __launch_bounds__(tc_threads(EG), 1)
           tc_fence_after();
           const uint32_t b_saddr = smem_u32(smem + (size_t)s * p.slot_bytes);
           const uint32_t a_taddr = tmem + tp.a_col0 + (uint32_t)s * 32u;
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t bdesc = smem_desc_sw128(b_saddr + (uint32_t)kk * 32u);
-            mma_ts(d_taddr, a_taddr + (uint32_t)kk * 8u, bdesc, idesc, (seg_first && kk == 0) ? 0u : 1u);
+            for (int kk = 0; kk < 4; ++kk) {
+              const uint64_t bdesc = smem_desc_sw128(b_saddr + (uint32_t)kk * 32u);
+              mma_ts(d_taddr, a_taddr + (uint32_t)kk * 8u, bdesc, idesc, (seg_first && kk == 0) ? 0u : 1u);
+            }
+            mma_commit(&stage_free[s]);
+            if (seg_last) mma_commit(&d_full[db * EG + (int)((w - w0) % EG)]);
           }
-          mma_commit(&stage_free[s]);
-          if (seg_last) mma_commit(&d_full[db * EG + (int)((w - w0) % EG)]);
+          __syncwarp();
         }
         if (++s == slots) {
           s = 0;

@@ -79,6 +79,15 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
+// True in one lane of the (converged) warp.  MMAs and commits are issued under this predicate
+// by a warp that walks its loop whole, not by a lane in a branch of its own: their operands
+// then stay in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // ------------------------------------------------------------------ CTA pairs (cta_group::2)
 // Tensor memory of both CTAs of a pair; a warp of each CTA takes part.
 __device__ __forceinline__ void tmem_alloc2(uint32_t* dst_smem, uint32_t ncols) {
@@ -121,30 +130,12 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(cbar)
       : "memory");
 }
+// Arrival on a barrier of the pair's other CTA (or this one).  What it orders is tensor memory
+// of this CTA, overwritten by the pair's MMAs, so the default scope (the CTA) is enough: no
+// data of one CTA is read by the other's threads.  At cluster scope the release is a fence
+// over the memory system.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cbar) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cbar) : "memory");
-}
-// Bounded wait whose phase may be completed from the other CTA of the cluster.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, uint64_t timeout_ns) {
-  const uint32_t a = smem_u32(bar);
-  auto done = [&] {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(a), "r"(parity)
-        : "memory");
-    return ok != 0;
-  };
-  if (done()) return true;
-  const uint64_t t0 = global_ns();
-  while (true) {
-    for (int i = 0; i < 64; ++i)
-      if (done()) return true;
-    if (global_ns() - t0 > timeout_ns) return false;
-  }
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cbar) : "memory");
 }
 
 }  // namespace sp
