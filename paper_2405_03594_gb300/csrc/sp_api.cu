@@ -32,7 +32,7 @@ constexpr int64_t kCudaCoreMaxM_int8 = 13;
 // Workspace of the documented contract, whatever kernel runs a batch of m rows.
 size_t workspace_bytes(const sp_matrix* h, int64_t m) {
   const size_t b = std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m));
-  return uses_dense(h, m) ? std::max(b, workspace_bytes_dense(h)) : b;
+  return uses_dense(h, m) ? std::max(b, workspace_bytes_dense(h, m)) : b;
 }
 
 bool uses_tensor_cores(const sp_matrix* h, int64_t m, sp_path path) {

@@ -124,28 +124,45 @@ struct DenseParams {
   int32_t tok;         // tokens per full tile
   int32_t tok_tiles;   // token tiles per 256 rows
   int64_t full;        // full tiles, tok tokens each
-  int64_t tiles;       // full tiles and the pieces of the rest
+  int64_t items;       // full tiles and the pieces of the rest, or tiles * split_k
   int32_t split;       // pieces per remaining tile, tok_piece tokens each
   int32_t tok_piece;
+  int32_t split_k;     // items that share a tile's K-tiles (1: none)
+  float* ws;           // split_k: partials [items][2 CTAs][tok][kRows]
+  int* cnt;            // split_k: arrival counters [tiles][2 CTAs]
   int32_t y_tma;
   int32_t stages;      // ring stages of stage_bytes: W's 16 KB, then a CTA's half of tok tokens of x
   uint32_t stage_bytes;
   uint64_t timeout_ns;
 };
 
-// Tile i of the work list: first row / 256, first token, tokens.  The first `full` tiles fill
-// whole waves of CTA pairs; the rest, less than a wave, is cut into narrower pieces so that
-// all pairs share it.
-__device__ __forceinline__ void tile_at(const DenseParams& p, int64_t i, int64_t* rt, int64_t* tok0, int* ntok) {
+// Item i of the work list: first row / 256, first token, tokens, K-tiles [t0, t1).  Without
+// split_k the first `full` items fill whole waves of CTA pairs with full tiles, and the rest,
+// less than a wave, is cut into narrower pieces so that all pairs share it.  With split_k (fewer
+// tiles than pairs, so one item per pair) a tile's K-tiles are shared by split_k items.
+struct Item {
+  int64_t rt, tok0;
+  int ntok, t0, t1;
+};
+__device__ __forceinline__ Item item_at(const DenseParams& p, int64_t i) {
+  Item it;
+  it.ntok = p.tok;
+  it.t0 = 0;
+  it.t1 = p.T;
   int64_t k = i, sub = 0;
-  *ntok = p.tok;
-  if (i >= p.full) {
+  if (p.split_k > 1) {
+    k = i / p.split_k;
+    const int part = (int)(i % p.split_k);
+    it.t0 = (int)((int64_t)part * p.T / p.split_k);
+    it.t1 = (int)((int64_t)(part + 1) * p.T / p.split_k);
+  } else if (i >= p.full) {
     k = p.full + (i - p.full) / p.split;
     sub = (i - p.full) % p.split;
-    *ntok = min(p.tok_piece, p.tok - (int)sub * p.tok_piece);
+    it.ntok = min(p.tok_piece, p.tok - (int)sub * p.tok_piece);
   }
-  *rt = k / p.tok_tiles;
-  *tok0 = (k % p.tok_tiles) * p.tok + sub * p.tok_piece;
+  it.rt = k / p.tok_tiles;
+  it.tok0 = (k % p.tok_tiles) * p.tok + sub * p.tok_piece;
+  return it;
 }
 
 __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
@@ -159,11 +176,10 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
   uint64_t* d_full = empty + kMaxStages;  // each CTA's: a tile's accumulators are complete
   uint64_t* d_empty = d_full + 2;      // leader's: both CTAs' epilogues have read the buffer
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(d_empty + 2);
+  volatile int* s_last = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_rank();
   const int64_t pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
-  const int T = p.T;
-
   if (tid == 0) {
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(&full[s], 1);
@@ -195,13 +211,11 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
       uint32_t ph = 0;
       bool dead = false;
       const uint32_t full0 = cluster_map(smem_u32(full), 0);
-      for (int64_t i = pair; i < p.tiles && !dead; i += pairs) {
-        int64_t rt, tok0;
-        int ntok;
-        tile_at(p, i, &rt, &tok0, &ntok);
-        const int wrow = (int)(rt * kTileRows + rank * kRows);  // (rows past the panel: clamped below)
-        const int xrow = (int)(tok0 + (int64_t)rank * (ntok / 2));
-        for (int t = 0; t < T; ++t) {
+      for (int64_t i = pair; i < p.items && !dead; i += pairs) {
+        const Item it = item_at(p, i);
+        const int wrow = (int)(it.rt * kTileRows + rank * kRows);  // (rows past the panel: clamped below)
+        const int xrow = (int)(it.tok0 + (int64_t)rank * (it.ntok / 2));
+        for (int t = it.t0; t < it.t1; ++t) {
           if (!mbar_wait(&empty[s], ph ^ 1u, p.timeout_ns)) {
             set_status(p.status, kStatusTimeout);
             dead = true;
@@ -239,11 +253,9 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
       uint32_t ph = 0;
       int64_t k = 0;  // tile number of this pair
       bool dead = false;
-      for (int64_t i = pair; i < p.tiles && !dead; i += pairs, ++k) {
-        int64_t rt, tok0;
-        int ntok;
-        tile_at(p, i, &rt, &tok0, &ntok);
-        const uint32_t idesc = idesc_bf16(kTileRows, ntok);
+      for (int64_t i = pair; i < p.items && !dead; i += pairs, ++k) {
+        const Item it = item_at(p, i);
+        const uint32_t idesc = idesc_bf16(kTileRows, it.ntok);
         const int db = (int)(k & 1);
         const uint32_t d = tmem + (uint32_t)db * kMaxTok;
         if (k >= 2 && !__all_sync(0xffffffffu, mbar_wait(&d_empty[db], (uint32_t)((k / 2 - 1) & 1), p.timeout_ns))) {
@@ -252,7 +264,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
           break;
         }
         tc_fence_after();
-        for (int t = 0; t < T; ++t) {
+        for (int t = it.t0; t < it.t1; ++t) {
           if (!__all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.timeout_ns))) {
             set_status(p.status, kStatusTimeout);
             dead = true;
@@ -264,9 +276,9 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
               mma_ss2(d, smem_desc_sw128(a + kk * 32u), smem_desc_sw128(a + kABytes + kk * 32u), idesc,
-                      (t > 0 || kk > 0) ? 1u : 0u);
+                      (t > it.t0 || kk > 0) ? 1u : 0u);
             mma_commit2(&empty[s]);
-            if (t == T - 1) mma_commit2(&d_full[db]);
+            if (t == it.t1 - 1) mma_commit2(&d_full[db]);
           }
           __syncwarp();
           if (++s == p.stages) {
@@ -287,10 +299,36 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
     int64_t k = 0;
     bool dead = false;
     pdl_wait();  // y belongs to the stream order
-    for (int64_t i = pair; i < p.tiles; i += pairs, ++k) {
-      int64_t rt, tok0;
-      int ntok;
-      tile_at(p, i, &rt, &tok0, &ntok);
+    const int etid = tid - kEpiWarp0 * 32;
+    // tokens tok .. tok + 31 of the CTA's rows from their sums v
+    auto store = [&](const float (&v)[32], int64_t tok, int64_t row0, float sc) {
+      const int64_t n = row0 + r;
+      if (p.y_tma) {
+        uint16_t* buf = stg + (size_t)(step & 1) * (kStgBytes / 2);
+        if (etid == 0) bulk_wait_read<1>();  // the store that last read it is done
+        named_bar_sync(1, 128);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) buf[j * kRows + r] = float_to_bf16_bits_rn(v[j] * sc);
+        fence_proxy_async_smem();
+        named_bar_sync(1, 128);
+        if (etid == 0) {
+          for (int b = 0; b < 32; b += kStgBox)
+            if (tok + b < p.M) tma_store_2d(&tmap_y, buf + b * kRows, (int)row0, (int)(tok + b));
+          bulk_commit();
+        }
+        ++step;
+      } else if (n < p.N) {
+        uint16_t* yp = p.y + tok * p.N + n;
+        const int nv = (int)imin64(32, p.M - tok);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          if (j < nv) *yp = float_to_bf16_bits_rn(v[j] * sc);
+          yp += p.N;
+        }
+      }
+    };
+    for (int64_t i = pair; i < p.items; i += pairs, ++k) {
+      const Item it = item_at(p, i);
       const int db = (int)(k & 1);
       if (!dead && !__all_sync(0xffffffffu, mbar_wait(&d_full[db], (uint32_t)((k / 2) & 1), p.timeout_ns))) {
         set_status(p.status, kStatusTimeout);
@@ -298,44 +336,85 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
       }
       // every epilogue warp takes the same branch: a warp that timed out keeps the barriers
       tc_fence_after();
-      const int64_t row0 = rt * kTileRows + rank * kRows;
-      const int64_t n = row0 + r;
-      const float sc = (p.scale && n < p.N) ? p.scale[n] : 1.f;
-      for (int c0 = 0; c0 < ntok; c0 += 32) {
-        uint32_t v[32];
+      const int64_t row0 = it.rt * kTileRows + rank * kRows;
+      const bool rows = row0 < p.N;  // the same for the whole CTA
+      const float sc = (p.scale && row0 + r < p.N) ? p.scale[row0 + r] : 1.f;
+      const int64_t part = (int64_t)kRows * p.tok;
+      float* wsp = p.ws + (i * 2 + rank) * part + r;
+      for (int c0 = 0; c0 < it.ntok; c0 += 32) {
+        float v[32];
         if (!dead) {
-          tmem_load32(tmem + (uint32_t)db * kMaxTok + lane_base + (uint32_t)c0, v);
+          uint32_t u[32];
+          tmem_load32(tmem + (uint32_t)db * kMaxTok + lane_base + (uint32_t)c0, u);
           tmem_load_wait();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(u[j]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = 0.f;
         }
-        if (c0 + 32 >= ntok) {  // the buffer is read: the issuer may start the tile after next
+        if (c0 + 32 >= it.ntok) {  // the buffer is read: the issuer may start the tile after next
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_remote(d_empty0 + 8u * db);
         }
-        if (row0 >= p.N) continue;  // the same for the whole CTA
-        if (p.y_tma) {
-          uint16_t* buf = stg + (size_t)(step & 1) * (kStgBytes / 2);
-          if (warp == kEpiWarp0 && lane == 0) bulk_wait_read<1>();  // the store that last read it is done
-          named_bar_sync(1, 128);
+        if (!rows) continue;
+        if (p.split_k == 1) {
+          store(v, it.tok0 + c0, row0, sc);
+        } else {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) buf[j * kRows + r] = float_to_bf16_bits_rn(__uint_as_float(v[j]) * sc);
-          fence_proxy_async_smem();
-          named_bar_sync(1, 128);
-          if (warp == kEpiWarp0 && lane == 0) {
-            for (int b = 0; b < 32; b += kStgBox)
-              if (tok0 + c0 + b < p.M) tma_store_2d(&tmap_y, buf + b * kRows, (int)row0, (int)(tok0 + c0 + b));
-            bulk_commit();
+          for (int j = 0; j < 32; ++j) __stcg(wsp + (int64_t)(c0 + j) * kRows, v[j]);
+        }
+      }
+      if (p.split_k == 1 || !rows) continue;
+      // the last of the tile's items to arrive adds up their partials in order
+      __threadfence();
+      named_bar_sync(1, 128);
+      const int64_t tile = i / p.split_k;
+      int* ctr = p.cnt + tile * 2 + rank;
+      if (etid == 0) *s_last = atomicAdd(ctr, 1) == p.split_k - 1 ? 1 : 0;
+      named_bar_sync(1, 128);
+      if (*s_last) {
+        __threadfence();
+        // a warp takes a token's 128 rows (four per lane), eight tokens at a time, so that 8
+        // or more 16-byte loads per lane are in flight: one CTA reads all of a tile's partials
+        const float4* src = reinterpret_cast<const float4*>(p.ws + (tile * p.split_k * 2 + rank) * part) + lane;
+        const int64_t n = row0 + 4 * lane;
+        float s4[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s4[j] = (p.scale && n + j < p.N) ? p.scale[n + j] : 1.f;
+        for (int tk = (warp & 3) * 8; tk < it.ntok; tk += 32) {
+          float4 v[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+          for (int q = 0; q < p.split_k; ++q) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float4 u = __ldcg(src + (2 * q * part + (int64_t)(tk + j) * kRows) / 4);
+              v[j].x += u.x, v[j].y += u.y, v[j].z += u.z, v[j].w += u.w;
+            }
           }
-          ++step;
-        } else if (n < p.N) {
-          uint16_t* yp = p.y + (tok0 + c0) * p.N + n;
-          const int nv = (int)imin64(32, p.M - (tok0 + c0));
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (j < nv) *yp = float_to_bf16_bits_rn(__uint_as_float(v[j]) * sc);
-            yp += p.N;
+          for (int j = 0; j < 8; ++j) {
+            const int64_t tok = it.tok0 + tk + j;
+            if (tok >= p.M) continue;
+            const uint32_t lo = (uint32_t)float_to_bf16_bits_rn(v[j].x * s4[0]) |
+                                ((uint32_t)float_to_bf16_bits_rn(v[j].y * s4[1]) << 16);
+            const uint32_t hi = (uint32_t)float_to_bf16_bits_rn(v[j].z * s4[2]) |
+                                ((uint32_t)float_to_bf16_bits_rn(v[j].w * s4[3]) << 16);
+            uint16_t* yp = p.y + tok * p.N + n;
+            if (p.N % 4 == 0) {
+              if (n < p.N) *reinterpret_cast<uint2*>(yp) = make_uint2(lo, hi);
+            } else {
+              if (n < p.N) yp[0] = (uint16_t)lo;
+              if (n + 1 < p.N) yp[1] = (uint16_t)(lo >> 16);
+              if (n + 2 < p.N) yp[2] = (uint16_t)hi;
+              if (n + 3 < p.N) yp[3] = (uint16_t)(hi >> 16);
+            }
           }
         }
+        if (etid == 0) atomicExch(ctr, 0);
       }
     }
     if (p.y_tma && warp == kEpiWarp0 && lane == 0) bulk_wait_all();
@@ -350,34 +429,52 @@ __global__ void __launch_bounds__(kDenseThreads, 1) __cluster_dims__(2, 1, 1)
 }
 
 // ------------------------------------------------------------------ host side
-// Work list for M tokens on `pairs` CTA pairs: the tile width (a multiple of 32 tokens) with
-// the least estimated time.  A tile costs per K-tile the larger of its tensor time, 2 clocks
-// per token, and its shared-memory traffic, 256 clocks for W's side (written and read) and one
-// per token for x's, and a fixed share for its start and end.
-void plan_tiles(const sp_matrix* h, int64_t M, int pairs, DenseParams* p) {
-  const int64_t rt = (h->RB + 1) / 2;
-  auto tile_cost = [&](int t) { return (double)h->T * std::max(2 * t, 256 + t) + 1500.0; };
+// Work list for M tokens on `pairs` CTA pairs: the tile width (a multiple of 32 tokens) and K
+// split with the least estimated time.  A tile costs per K-tile the largest of its tensor time,
+// 2 clocks per token, its shared-memory traffic, 256 clocks for W's side (written and read) and
+// one per token for x's, and ~430 clocks of issue and barriers, and a fixed share for its start
+// and end.  Splitting K (at least 8 K-tiles per item) pays where the tiles would leave pairs
+// idle; its partial sums are written once and read by one CTA per tile (~600 clocks per 32
+// tokens and part).  Measured at 70 %, unsplit / split: 4096 x 4096 24.6 / 20.4 us at 64 tokens,
+// 4096 x 11008 55.4 / 37.1 at 64, 55.6 / 41.8 at 128.
+void plan_items(const sp_matrix* h, int64_t M, int pairs, DenseParams* p) {
+  const int64_t rt = (h->RB + 1) / 2, T = h->T;
+  auto cost = [&](int64_t kt, int t) { return (double)kt * std::max({2 * t, 256 + t, 430}) + 1500.0; };
   double best = 0;
+  auto take = [&](double c) {
+    if (best != 0 && c >= best) return false;
+    best = c;
+    return true;
+  };
   for (int t = 32; t <= kMaxTok; t += 32) {
     const int64_t tt = (M + t - 1) / t;
     const int64_t total = rt * tt, waves = total / pairs, rest = total - waves * pairs;
-    double cost = (double)waves * tile_cost(t);
+    double c = (double)waves * cost(T, t);
     int split = 1, piece = t;
     if (rest > 0) {
       const int units = t / 32;
       const int want = (int)std::min<int64_t>(pairs / rest, units);
       piece = (units + want - 1) / want * 32;
       split = (t + piece - 1) / piece;
-      cost += tile_cost(piece);
+      c += cost(T, piece);
     }
-    if (best == 0 || cost < best) {
-      best = cost;
+    if (take(c)) {
       p->tok = t;
       p->tok_tiles = (int32_t)tt;
       p->full = waves * pairs;
       p->split = split;
       p->tok_piece = piece;
-      p->tiles = p->full + rest * split;
+      p->items = p->full + rest * split;
+      p->split_k = 1;
+    }
+    const int64_t sk = std::min<int64_t>(pairs / total, T / 8);
+    if (sk >= 2 && take(cost((T + sk - 1) / sk, t) + 3000.0 + 600.0 * (double)(sk * (t / 32)))) {
+      p->tok = p->tok_piece = t;
+      p->tok_tiles = (int32_t)tt;
+      p->full = 0;
+      p->split = 1;
+      p->items = total * sk;
+      p->split_k = (int32_t)sk;
     }
   }
 }
@@ -409,34 +506,42 @@ size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
 }  // namespace
 
-// Against linear_tc_kernel, measured at 70 %: from 33 tokens on where the matrix is small (4096 x
-// 4096 30.8 us against 34.6 at M = 64, 31.6 / 102 at 256; 1003 x 1096 11.7 / 65), later where the
-// scratch is much traffic for few tokens (q/k/v INT8 45 / 43 at 33, 50 / 83 at 256; down 71 / 67 at
-// 128, 72 / 90 at 192; gate/up 90 / 82 at 256, 102 / 121 at 384, 233 / 377 at 2048).  A matrix of
-// fewer chunks than SMs keeps the one launch.
+// Against linear_tc_kernel, measured at 70 %: from 33 tokens on where the matrix is small or of
+// middling size (4096 x 4096 20 us against 33 at M = 64, 25 / 101 at 256; 1003 x 1096 10 / 63 at 64;
+// down 37 / 40 at 33, 53 / 111 at 256), later where the scratch is much traffic for few tokens
+// (q/k/v 39 / 36 at 64, 41 / 50 at 128; gate/up 79 / 59 at 128, 83 / 81 at 256, 94 / 120 at 384,
+// 218 / 376 at 2048).  A matrix of fewer chunks than SMs keeps the one launch.
 bool uses_dense(const sp_matrix* h, int64_t M) {
   const int64_t C = (int64_t)h->RB * h->T, rows = (int64_t)h->RB * kRows;
   if (C < h->num_sms || M > (int64_t)1 << 24 || (int64_t)h->T * rows >= (int64_t)1 << 31) return false;
-  return M > kMmaMaxRows && M >= (C <= 2500 ? 0 : C / 40);
+  return M > kMmaMaxRows && 24 * M >= C - 5000;
 }
 
-size_t workspace_bytes_dense(const sp_matrix* h) {
-  return ws_counter_bytes(h->num_sms) + round256((size_t)h->T * h->RB * kRows * 128);
+namespace {
+size_t scratch_bytes(const sp_matrix* h) { return round256((size_t)h->T * h->RB * kRows * 128); }
+}  // namespace
+
+// [arrival counters][expanded matrix][split-K partials: two CTAs of at most num_sms / 2 items]
+size_t workspace_bytes_dense(const sp_matrix* h, int64_t M) {
+  const size_t tok = (size_t)std::min<int64_t>(kMaxTok, (M + 31) / 32 * 32);
+  return ws_counter_bytes(h->num_sms) + scratch_bytes(h) + (size_t)(h->num_sms / 2) * 2 * kRows * tok * sizeof(float);
 }
 
 sp_status launch_linear_dense(const sp_matrix* h, const uint16_t* x, int64_t M, uint16_t* y, void* ws, size_t ws_bytes,
                               cudaStream_t stream) {
-  if (!ws || ws_bytes < workspace_bytes_dense(h)) return SP_ERR_WORKSPACE;
+  if (!ws || ws_bytes < workspace_bytes_dense(h, M)) return SP_ERR_WORKSPACE;
   const int64_t rows = (int64_t)h->RB * kRows;
   PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   sp_status st = tensor_map_encoder(&encode);
   if (st != SP_OK) return st;
-  const int pairs = resident_pairs(h->device);
+  const int pairs = std::min(resident_pairs(h->device), h->num_sms / 2);
   if (pairs < 1) return SP_ERR_CUDA;
 
   // the scratch follows the arrival counters, which stay zero for the other kernels
   uint8_t* scratch = static_cast<uint8_t*>(ws) + ws_counter_bytes(h->num_sms);
   DenseParams p{};
+  p.cnt = static_cast<int*>(ws);
+  p.ws = reinterpret_cast<float*>(scratch + scratch_bytes(h));
   p.y = y;
   p.scale = h->d_scale;
   p.status = device_status_ptr();
@@ -446,7 +551,7 @@ sp_status launch_linear_dense(const sp_matrix* h, const uint16_t* x, int64_t M, 
   p.T = h->T;
   p.y_tma = h->N % 8 == 0 ? 1 : 0;
   p.timeout_ns = wait_timeout_ns();
-  plan_tiles(h, M, pairs, &p);
+  plan_items(h, M, pairs, &p);
   p.stage_bytes = (uint32_t)(kABytes + p.tok / 2 * 128);  // a multiple of 2 KB
   p.stages = (int32_t)std::min<uint32_t>(kMaxStages, kRingBytes / p.stage_bytes);
 
@@ -484,7 +589,7 @@ sp_status launch_linear_dense(const sp_matrix* h, const uint16_t* x, int64_t M, 
                                                            reinterpret_cast<uint4*>(scratch), p.timeout_ns, p.status);
   if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(2 * std::min<int64_t>(pairs, p.tiles)));
+  cfg.gridDim = dim3((unsigned)(2 * std::min<int64_t>(pairs, p.items)));
   cfg.blockDim = dim3(kDenseThreads);
   cfg.dynamicSmemBytes = kDenseSmem;
   cfg.stream = stream;
