@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(kRows) expand_kernel(const uint8_t* __restrict
   const int64_t c = blockIdx.x;
   const int64_t rb = c / T, t = c % T;
   const int tid = threadIdx.x, lane = tid & 31, q = tid >> 5;
+  pdl_launch_dependents();  // the product's CTAs may set up while the last chunks are expanded
   if (tid == 0) {
     mbar_init(&bar, 1);
     fence_barrier_init();
@@ -73,6 +74,7 @@ __global__ void __launch_bounds__(kRows) expand_kernel(const uint8_t* __restrict
     reinterpret_cast<uint2*>(s_start)[tid] = make_uint2(e0 * ES, (e0 + (uint32_t)plo) * ES);
   }
   __syncwarp();
+  pdl_wait();  // the scratch belongs to the stream order, the weights do not
   const int seg = lane & 7, half = seg >> 2, sh = 8 * (seg & 3);
   const uint32_t below = (1u << sh) - 1u;
   const uint32_t vbase = smem_u32(chunk) + kMaskBytes;
@@ -510,10 +512,10 @@ size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 // middling size (4096 x 4096 20 us against 33 at M = 64, 25 / 101 at 256; 1003 x 1096 10 / 63 at 64;
 // down 37 / 40 at 33, 53 / 111 at 256), later where the scratch is much traffic for few tokens
 // (q/k/v 39 / 36 at 64, 41 / 50 at 128; gate/up 79 / 59 at 128, 83 / 81 at 256, 94 / 120 at 384,
-// 218 / 376 at 2048).  A matrix of fewer chunks than SMs keeps the one launch.
+// 218 / 376 at 2048).  A matrix of a few chunks keeps the one launch.
 bool uses_dense(const sp_matrix* h, int64_t M) {
   const int64_t C = (int64_t)h->RB * h->T, rows = (int64_t)h->RB * kRows;
-  if (C < h->num_sms || M > (int64_t)1 << 24 || (int64_t)h->T * rows >= (int64_t)1 << 31) return false;
+  if (C < 16 || M > (int64_t)1 << 24 || (int64_t)h->T * rows >= (int64_t)1 << 31) return false;
   return M > kMmaMaxRows && 24 * M >= C - 5000;
 }
 
@@ -585,24 +587,31 @@ sp_status launch_linear_dense(const sp_matrix* h, const uint16_t* x, int64_t M, 
 
   const int64_t C = (int64_t)h->RB * h->T;
   auto ek = h->esize == 2 ? expand_kernel<2> : expand_kernel<1>;
-  ek<<<(unsigned)C, kRows, (size_t)h->max_chunk, stream>>>(h->d_buf, h->d_off, h->d_qidx, h->T, rows,
-                                                           reinterpret_cast<uint4*>(scratch), p.timeout_ns, p.status);
-  if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(2 * std::min<int64_t>(pairs, p.items)));
-  cfg.blockDim = dim3(kDenseThreads);
-  cfg.dynamicSmemBytes = kDenseSmem;
-  cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  // after an in-place weight update the expansion waits for the whole previous grid
+  attr[0].val.programmaticStreamSerializationAllowed = h->weights_written ? 0 : 1;
+  cfg.gridDim = dim3((unsigned)C);
+  cfg.blockDim = dim3(kRows);
+  cfg.dynamicSmemBytes = (size_t)h->max_chunk;
+  cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, dense_kernel, p, map_w, map_x, map_y) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, ek, h->d_buf, h->d_off, h->d_qidx, h->T, rows, reinterpret_cast<uint4*>(scratch),
+                         p.timeout_ns, p.status) != cudaSuccess) {
     cudaGetLastError();
     return SP_ERR_CUDA;
   }
   h->weights_written = 0;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3((unsigned)(2 * std::min<int64_t>(pairs, p.items)));
+  cfg.blockDim = dim3(kDenseThreads);
+  cfg.dynamicSmemBytes = kDenseSmem;
+  if (cudaLaunchKernelEx(&cfg, dense_kernel, p, map_w, map_x, map_y) != cudaSuccess) {
+    cudaGetLastError();
+    return SP_ERR_CUDA;
+  }
   return SP_OK;
 }
 

@@ -23,7 +23,7 @@ def _matrix(sp, N, K, int8, g):
     return (W, mask, None), sp.compress(gu.bf16_to_dev(W), gu.u8_to_dev(mask))
 
 
-@pytest.mark.parametrize("N,K,M", [(1150, 1096, 33), (2048, 1024, 300), (1500, 2056, 513), (19520, 64, 70),
+@pytest.mark.parametrize("N,K,M", [(256, 512, 40), (1150, 1096, 33), (2048, 1024, 300), (1500, 2056, 513), (19520, 64, 70),
                                    (6000, 328, 2049), (128, 11008, 100)])
 @pytest.mark.parametrize("int8", [False, True])
 def test_integer_sums_bit_exact(oracle, N, K, M, int8):
