@@ -32,8 +32,8 @@
 //                    at a time.
 // At the end of its K-tiles a CTA adds its warps' sums in warp order in shared memory (on the
 // ring, which is idle by then); the cluster's CTAs then each sum a share of the tokens over
-// all ranks in rank order (distributed shared memory) and write y through the launch's output
-// epilogue.  All orders are fixed: results are bitwise repeatable.
+// all ranks in rank order (distributed shared memory: pushed to the owner by the eight-warp form
+// up to 8 tokens, read by it otherwise) and write y through the launch's output epilogue.  All orders are fixed: results are bitwise repeatable.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -60,7 +60,7 @@ struct MmaParams {
   int32_t T, M;
   int32_t cluster;     // CTAs per row block
   int32_t slots;
-  uint32_t chunk_region, ring_off, tab_off, bar_off;
+  uint32_t chunk_region, ring_off, tab_off, bar_off, rx_off;
   int32_t epi;
   int32_t early;       // release the next launch as soon as this one's inputs are ready
   uint64_t timeout_ns;
@@ -134,6 +134,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
   constexpr int R = RW / 32;               // rows per lane in the scan
   constexpr int kTiles = RW / 16;          // 16-row tiles of a warp
   constexpr uint32_t kXBytes = NT * 1024u;
+  constexpr bool kPush = NT == 1 && CW == 8;  // how the cluster's sums meet (at the end)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int slots = p.slots;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.bar_off);
@@ -155,6 +156,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
     fence_barrier_init();
   }
   __syncthreads();
+  if (kPush && p.cluster > 1) cluster_arrive_relaxed();  // this CTA runs: its shared memory may be written
 
   if (warp == CW) {
     // ------------------------------------------------------------ producer
@@ -360,13 +362,39 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
     }
     return;
   }
-  if constexpr (kGroups > 1) {
-    for (int m = m0; m < M; m += kStep) {
-      float v = comb[m * kRows + rr];
+  auto cta_sum = [&](int m) {
+    float v = comb[m * kRows + rr];
 #pragma unroll
-      for (int q = 1; q < kGroups; ++q) v += comb[(q * M + m) * kRows + rr];
-      comb[m * kRows + rr] = v;
+    for (int q = 1; q < kGroups; ++q) v += comb[(q * M + m) * kRows + rr];
+    return v;
+  };
+  if constexpr (kPush) {
+    // Few tokens: rank m % S owns token m, and every CTA stores its sum of it straight into the
+    // owner's receive area ([tokens owned][S][kRows] floats, apart from the ring, which the
+    // owner may still be using): one cluster barrier at the end.  Reading the sums from the
+    // other CTAs' memory takes one before, so that they are there, and one after, so that they
+    // stay.  Measured, read / pushed: 512 x 11008 7.6 / 7.2 us, down at 80 % 17.4 / 16.9, q/k/v
+    // at 50 % 21.6 / 21.0 (M = 4).  The four-warp form reads: its grids fill every CTA slot, and
+    // how the CTAs leave decides how evenly the next launch's come in (gate/up 28.1 us read at
+    // M = 3 and 4, pushed 30.0 and 26.9).
+    const int S = p.cluster;
+    const uint32_t rx = smem_u32(smem + p.rx_off) + 4u * (uint32_t)(rank * kRows + rr);
+    cluster_wait();
+    for (int m = m0; m < M; m += kStep)
+      st_cluster_f32(cluster_map(rx + 4u * (uint32_t)(m / S * S * kRows), (uint32_t)(m % S)), cta_sum(m));
+    cluster_arrive_release();
+    cluster_wait();
+    const float* got = reinterpret_cast<const float*>(smem + p.rx_off) + rr;
+    for (int m = rank + m0 * S; m < M; m += kStep * S) {
+      float v = 0.f;
+#pragma unroll 4
+      for (int q = 0; q < S; ++q) v += got[(m / S * S + q) * kRows];
+      write_one(p, row, m, v, sc);
     }
+    return;
+  }
+  if constexpr (kGroups > 1) {
+    for (int m = m0; m < M; m += kStep) comb[m * kRows + rr] = cta_sum(m);
   }
   cluster_sync_all();
   const uint32_t mine = smem_u32(comb) + 4u * (uint32_t)rr;
@@ -386,7 +414,7 @@ struct MmaChoice {
 };
 struct MmaPlan {
   int slots, cluster;
-  uint32_t chunk_region, ring_off, tab_off, bar_off;
+  uint32_t chunk_region, ring_off, tab_off, bar_off, rx_off;
   size_t smem;
 };
 
@@ -461,7 +489,9 @@ bool mma_plan(const sp_matrix* h, int M, const MmaChoice& c, int occ, int min_sl
   pl->chunk_region = (uint32_t)((h->max_chunk + 127) / 128 * 128);
   const size_t budget = ((size_t)(227 * 1024) / occ - 1024) / 128 * 128;  // all of it is asked for
   const size_t tab = (size_t)c.cw * c.rw * 16;
-  const size_t ctl = (size_t)kMaxSlots * (8 + 8 + 8 + 4);
+  const int S = pl->cluster;
+  const size_t rx = c.nt == 1 && c.cw == 8 && S > 1 ? (size_t)(M + S - 1) / S * S * kRows * sizeof(float) : 0;  // receive area
+  const size_t ctl = (size_t)kMaxSlots * (8 + 8 + 8 + 4) + rx;
   const size_t per_slot = (size_t)c.nt * 1024 + pl->chunk_region;
   if (budget < tab + ctl + min_slots * per_slot) return false;
   const int items = (h->T + pl->cluster - 1) / pl->cluster;
@@ -472,6 +502,7 @@ bool mma_plan(const sp_matrix* h, int M, const MmaChoice& c, int occ, int min_sl
   const size_t ring_end = std::max<size_t>(pl->ring_off + (size_t)pl->slots * pl->chunk_region, (sums + 127) / 128 * 128);
   pl->tab_off = (uint32_t)ring_end;
   pl->bar_off = (uint32_t)(ring_end + tab);
+  pl->rx_off = (uint32_t)(pl->bar_off + ctl - rx);
   if (pl->bar_off + ctl > budget) return false;
   // The whole share of shared memory, whatever the chunks need: CTAs of consecutive launches
   // then fit the holes that each other's leave.  Sizes following the largest chunk cost 33.2
@@ -576,6 +607,7 @@ sp_status launch_linear_mma(const sp_matrix* h, const uint16_t* x, int64_t M, ui
   p.ring_off = pl.ring_off;
   p.tab_off = pl.tab_off;
   p.bar_off = pl.bar_off;
+  p.rx_off = pl.rx_off;
   p.epi = epi;
   p.early = overlaps((int64_t)h->RB * pl.cluster, (int64_t)c.occ * h->num_sms) ? 1 : 0;
   p.timeout_ns = wait_timeout_ns();
