@@ -31,11 +31,11 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t v) {
 }
 
 // Also writes the chunk's quarter index (kept entries before rows 32, 64 and 96, and in the
-// whole chunk; 16 bits each) and raises *max_quarter to its largest quarter count.  Warp q
-// takes rows 32q .. 32q+31, four at a time; a lane packs eight columns of one row.
+// whole chunk; 16 bits each).  Warp q takes rows 32q .. 32q+31, four at a time; a lane packs
+// eight columns of one row.
 __global__ void __launch_bounds__(kRows) count_kernel(const uint8_t* __restrict__ mask, int64_t N, int64_t K, int T,
-                                                      uint8_t* __restrict__ masks_out, int* __restrict__ cnt,
-                                                      uint64_t* __restrict__ qidx, int* __restrict__ max_quarter) {
+                                                      uint8_t* __restrict__ masks_out,
+                                                      uint64_t* __restrict__ qidx) {
   __shared__ int s_q[kRows / 32];
   const int64_t c = blockIdx.x;
   const int64_t rb = c / T, t = c % T;
@@ -61,25 +61,28 @@ __global__ void __launch_bounds__(kRows) count_kernel(const uint8_t* __restrict_
   __syncthreads();
   if (threadIdx.x == 0) {
     const int a = s_q[0], b = a + s_q[1], d = b + s_q[2], total = d + s_q[3];
-    cnt[c] = total;
     qidx[c] = (uint64_t)a | ((uint64_t)b << 16) | ((uint64_t)d << 32) | ((uint64_t)total << 48);
-    atomicMax(max_quarter, max(max(s_q[0], s_q[1]), max(s_q[2], s_q[3])));
   }
 }
 
-// meta[0] = total bytes, meta[1] = largest chunk, meta[2] = kept entries.  Thread i owns the
+// meta[0] = total bytes, meta[1] = largest chunk, meta[2] = kept entries, meta[3] = most kept
+// entries in a quarter, all from the chunks' quarter indices.  Thread i owns the
 // run of ceil(C / 1024) chunks from i * ceil(C / 1024): one pass sums the runs, one block scan
 // gives their starts, a second pass writes the offsets.
-__global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ cnt, int64_t C, int esize,
+__global__ void __launch_bounds__(1024) scan_kernel(const uint64_t* __restrict__ qidx, int64_t C, int esize,
                                                     uint64_t* __restrict__ off, uint64_t* __restrict__ meta) {
   __shared__ uint64_t s_warp[32];
   __shared__ uint64_t s_max[32], s_nnz[32];
+  __shared__ uint32_t s_quarter[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t run = (C + 1023) / 1024;
   const int64_t c0 = imin64(run * threadIdx.x, C), c1 = imin64(c0 + run, C);
   uint64_t sum = 0, mx = 0, nnz = 0;
+  uint32_t quarter = 0;
   for (int64_t i = c0; i < c1; ++i) {
-    const uint64_t kept = (uint64_t)__ldg(cnt + i);
+    const uint64_t qi = qidx[i], kept = qi >> 48;
+    const uint32_t a = (uint32_t)(qi & 0xffffu), b = (uint32_t)(qi >> 16) & 0xffffu, d = (uint32_t)(qi >> 32) & 0xffffu;
+    quarter = max(quarter, max(max(a, b - a), max(d - b, (uint32_t)kept - d)));
     const uint64_t sz = (kMaskBytes + kept * esize + 15) / 16 * 16;
     mx = max(mx, sz);
     nnz += kept;
@@ -96,7 +99,9 @@ __global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ cnt,
     mx = max(mx, __shfl_down_sync(0xffffffffu, mx, d));
     nnz += __shfl_down_sync(0xffffffffu, nnz, d);
   }
+  quarter = __reduce_max_sync(0xffffffffu, quarter);
   if (lane == 0) {
+    s_quarter[warp] = quarter;
     s_max[warp] = mx;
     s_nnz[warp] = nnz;
   }
@@ -105,11 +110,13 @@ __global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ cnt,
   for (int w = 0; w < warp; ++w) o += s_warp[w];
   for (int64_t i = c0; i < c1; ++i) {
     off[i] = o;
-    o += (kMaskBytes + (uint64_t)__ldg(cnt + i) * esize + 15) / 16 * 16;
+    o += (kMaskBytes + (qidx[i] >> 48) * esize + 15) / 16 * 16;
   }
   if (threadIdx.x == 0) {
     uint64_t all = 0, a = 0, b = 0;
+    uint32_t most = 0;
     for (int w = 0; w < 32; ++w) {
+      most = max(most, s_quarter[w]);
       all += s_warp[w];
       a = max(a, s_max[w]);
       b += s_nnz[w];
@@ -118,6 +125,7 @@ __global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ cnt,
     meta[0] = all;
     meta[1] = a;
     meta[2] = b;
+    meta[3] = most;
   }
 }
 
@@ -327,6 +335,10 @@ __global__ void __launch_bounds__(kRows) decompress_kernel(const uint8_t* __rest
 
 }  // namespace
 
+namespace {
+size_t round256(size_t b) { return (b + 255) / 256 * 256; }
+}  // namespace
+
 void* dev_alloc(const sp_matrix* h, size_t bytes) {
   if (bytes == 0) bytes = 16;
   if (h->alloc) return h->alloc(bytes, h->ctx);
@@ -344,6 +356,21 @@ void dev_free(const sp_matrix* h, void* p) {
     h->free_fn(p, h->ctx);
   else
     cudaFree(p);
+}
+
+size_t index_bytes(const sp_matrix* h) {
+  const size_t C = (size_t)h->RB * h->T;
+  return round256((C + 1) * sizeof(uint64_t)) + round256(C * sizeof(uint64_t)) +
+         (h->dtype == SP_INT8 ? (size_t)h->N * sizeof(float) : 0);
+}
+
+bool alloc_index(sp_matrix* h) {
+  const size_t C = (size_t)h->RB * h->T;
+  uint8_t* p = (uint8_t*)dev_alloc(h, index_bytes(h));
+  h->d_off = (uint64_t*)p;
+  h->d_qidx = p ? (uint64_t*)(p + round256((C + 1) * sizeof(uint64_t))) : nullptr;
+  h->d_scale = p && h->dtype == SP_INT8 ? (float*)((uint8_t*)h->d_qidx + round256(C * sizeof(uint64_t))) : nullptr;
+  return p != nullptr;
 }
 
 sp_status launch_compress(const void* w, const uint8_t* mask, int64_t N, int64_t K, sp_dtype dt, const float* scale,
@@ -364,24 +391,16 @@ sp_status launch_compress(const void* w, const uint8_t* mask, int64_t N, int64_t
   const int64_t C = (int64_t)h->RB * h->T;
 
   sp_status st = SP_OK;
-  uint64_t* d_masks = (uint64_t*)dev_alloc(h, (size_t)C * kMaskBytes);
-  int* d_cnt = (int*)dev_alloc(h, (size_t)C * sizeof(int));
-  uint64_t* d_meta = (uint64_t*)dev_alloc(h, 4 * sizeof(uint64_t));
-  h->d_off = (uint64_t*)dev_alloc(h, (size_t)(C + 1) * sizeof(uint64_t));
-  h->d_qidx = (uint64_t*)dev_alloc(h, (size_t)C * sizeof(uint64_t));
+  // scratch for the call: the masks, then the totals
+  uint64_t* d_masks = (uint64_t*)dev_alloc(h, (size_t)C * kMaskBytes + 4 * sizeof(uint64_t));
+  uint64_t* d_meta = d_masks ? d_masks + (size_t)C * kRows : nullptr;
   uint64_t meta[4] = {0, 0, 0, 0};
-  if (!d_masks || !d_cnt || !d_meta || !h->d_off || !h->d_qidx) {
+  if (!d_masks || !alloc_index(h)) {
     st = SP_ERR_OUT_OF_MEMORY;
     goto fail;
   }
-  // meta[3] holds the largest quarter count (count_kernel's atomicMax target)
-  if (cudaMemsetAsync(d_meta, 0, 4 * sizeof(uint64_t), stream) != cudaSuccess) {
-    st = SP_ERR_CUDA;
-    goto fail;
-  }
-  count_kernel<<<(unsigned)C, kRows, 0, stream>>>(mask, N, K, h->T, reinterpret_cast<uint8_t*>(d_masks), d_cnt,
-                                                   h->d_qidx, reinterpret_cast<int*>(d_meta + 3));
-  scan_kernel<<<1, 1024, 0, stream>>>(d_cnt, C, h->esize, h->d_off, d_meta);
+  count_kernel<<<(unsigned)C, kRows, 0, stream>>>(mask, N, K, h->T, reinterpret_cast<uint8_t*>(d_masks), h->d_qidx);
+  scan_kernel<<<1, 1024, 0, stream>>>(h->d_qidx, C, h->esize, h->d_off, d_meta);
   if (cudaGetLastError() != cudaSuccess) {
     st = SP_ERR_CUDA;
     goto fail;
@@ -401,11 +420,6 @@ sp_status launch_compress(const void* w, const uint8_t* mask, int64_t N, int64_t
     goto fail;
   }
   if (dt == SP_INT8) {
-    h->d_scale = (float*)dev_alloc(h, (size_t)N * sizeof(float));
-    if (!h->d_scale) {
-      st = SP_ERR_OUT_OF_MEMORY;
-      goto fail;
-    }
     if (cudaMemcpyAsync(h->d_scale, scale, (size_t)N * sizeof(float), cudaMemcpyDeviceToDevice, stream) !=
         cudaSuccess) {
       st = SP_ERR_CUDA;
@@ -423,8 +437,6 @@ sp_status launch_compress(const void* w, const uint8_t* mask, int64_t N, int64_t
     goto fail;
   }
   dev_free(h, d_masks);
-  dev_free(h, d_cnt);
-  dev_free(h, d_meta);
   h->magic = SP_MAGIC;
   *out = h;
   return SP_OK;
@@ -433,12 +445,8 @@ fail:
   cudaStreamSynchronize(stream);
   cudaGetLastError();
   dev_free(h, d_masks);
-  dev_free(h, d_cnt);
-  dev_free(h, d_meta);
   dev_free(h, h->d_off);
-  dev_free(h, h->d_qidx);
   dev_free(h, h->d_buf);
-  dev_free(h, h->d_scale);
   delete h;
   return st;
 }

@@ -24,7 +24,7 @@ struct sp_matrix {
   uint64_t max_chunk;
   uint32_t max_quarter;  // most kept entries in one 32-row quarter of a chunk
   uint8_t* d_buf;
-  uint64_t* d_off;
+  uint64_t* d_off;       // one allocation holds d_off, d_qidx and d_scale (alloc_index)
   uint64_t* d_qidx;      // per chunk: kept entries before rows 32, 64, 96 and in all 128 rows
                          // (16 bits each, low to high), derived from the masks at compression
   float* d_scale;
@@ -325,6 +325,10 @@ sp_status launch_linear_dense(const sp_matrix* h, const uint16_t* x, int64_t M, 
 sp_status tensor_map_encoder(PFN_cuTensorMapEncodeTiled_v12000* out);  // cuTensorMapEncodeTiled, looked up once
 int* device_status_ptr();            // this device's status word (device address)
 uint64_t wait_timeout_ns();          // bounded-wait limit for kernels
+// d_off, d_qidx and (INT8) d_scale of a handle whose sizes are set, as one allocation of
+// index_bytes at d_off; false if the allocator has none.
+size_t index_bytes(const sp_matrix* h);
+bool alloc_index(sp_matrix* h);
 void* dev_alloc(const sp_matrix* h, size_t bytes);
 void dev_free(const sp_matrix* h, void* p);
 
