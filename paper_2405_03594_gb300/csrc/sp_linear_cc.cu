@@ -880,7 +880,12 @@ bool cc_plan(const sp_matrix* h, int Mt, int S, int occ, CcPlan* pl) {
                              4 * (size_t)pl->slots + 15) /
                             16 * 16);
   pl->part_off = pl->comb_off + (uint32_t)(pl->kind == 1 ? comb_bytes : 0);
-  pl->smem = pl->part_off + part_bytes;
+  // at least the whole share of shared memory, whatever the chunks need: CTAs of consecutive
+  // launches then fit the holes that each other's leave (a decode step of four layers at M = 1
+  // took 263.6 us, or 269 to 278 where matrices' largest chunks differ)
+  pl->smem = std::max<size_t>(pl->part_off + part_bytes, occ == kCtasPerSmM1    ? kSmemBudgetM1
+                                                         : occ == kCtasPerSmM1b ? kSmemBudgetM1b
+                                                                                : kSmemBudget);
   return true;
 }
 
