@@ -57,11 +57,13 @@ __device__ __forceinline__ uint32_t expand_word_u8(uint32_t m, uint32_t& pa) {
 // Two signed bytes (bits 0-7 and 16-23 of w, zero elsewhere) as bf16x2, exactly.  128 plus the
 // byte's low seven bits is the bf16 0x4300 | low7, and its sign bit, weight -128, turns the
 // 128 = 0x4300 to subtract into 256 = 0x4380: one subtraction of two exact bf16 leaves q.
-__device__ __forceinline__ uint32_t i8x2_to_bf16x2(uint32_t w) {
-  const uint32_t a = (w & 0x007f007fu) | 0x43004300u, b = (w & 0x00800080u) | 0x43004300u;
+__device__ __forceinline__ uint32_t sub_bf16x2(uint32_t a, uint32_t b) {
   uint32_t o;
   asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(o) : "r"(a), "r"(b));
   return o;
+}
+__device__ __forceinline__ uint32_t i8x2_to_bf16x2(uint32_t w) {
+  return sub_bf16x2((w & 0x007f007fu) | 0x43004300u, (w & 0x00800080u) | 0x43004300u);
 }
 
 }  // namespace sp

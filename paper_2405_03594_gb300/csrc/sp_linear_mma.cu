@@ -60,7 +60,7 @@ struct MmaParams {
   int32_t T, M;
   int32_t cluster;     // CTAs per row block
   int32_t slots;
-  uint32_t chunk_region, ring_off, tab_off, bar_off, rx_off;
+  uint32_t chunk_region, ring_off, tab_off, bar_off, lut_off, rx_off;
   int32_t epi;
   int32_t early;       // release the next launch as soon as this one's inputs are ready
   uint64_t timeout_ns;
@@ -82,26 +82,50 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Two columns as bf16x2 from a row's value stream (columns 2P, 2P + 1 of the mask piece m).
-template <int ES, int P>
-__device__ __forceinline__ uint32_t expand2(uint32_t m, uint32_t& pa) {
-  if constexpr (ES == 2)
-    return expand_word_bf16<1u << (2 * P), 2u << (2 * P)>(m, pa);
-  else
-    return i8x2_to_bf16x2(expand_word_u8<1u << (2 * P), 2u << (2 * P)>(m, pa));
+// Four columns (bits 4S .. 4S + 3 of the mask piece m) as two bf16x2 from a row's value stream
+// at shared address pa, which advances.
+//
+// bf16: a predicated load per column (sp_expand.cuh).  INT8: four values are one word, so the
+// four columns' bytes are placed by a single byte permutation of the next four stream bytes (two
+// aligned words and a funnel shift), its selector and the kept count looked up by the four mask
+// bits in a 16-word table that no two lanes' different words share a bank of.  That takes 19
+// instructions where four byte loads, their tests and increments took 24: gate/up 34.1 -> 30.5 us
+// at M = 4, 70 %.
+template <int ES, int S>
+__device__ __forceinline__ void expand4(uint32_t m, uint32_t& pa, uint32_t lut, uint32_t& c01, uint32_t& c23) {
+  if constexpr (ES == 2) {
+    c01 = expand_word_bf16<1u << (4 * S), 2u << (4 * S)>(m, pa);
+    c23 = expand_word_bf16<4u << (4 * S), 8u << (4 * S)>(m, pa);
+  } else {
+    const uint32_t e = lds32(lut + ((S == 0 ? m << 2 : m >> (4 * S - 2)) & 0x3cu));
+    const uint32_t a = pa & ~3u;
+    const uint32_t win = __funnelshift_r(lds32(a), lds32(a + 4), pa << 3);
+    const uint32_t x = __byte_perm(win, 0u, e);
+    pa += e >> 16;
+    // byte q -> 0x43qq: 128 + its low seven bits, minus 128 or (sign bit) 256, as i8x2_to_bf16x2
+    const uint32_t y0 = __byte_perm(x, 0x43434343u, 0x4140u), y1 = __byte_perm(x, 0x43434343u, 0x4342u);
+    c01 = sub_bf16x2(y0 & 0xff7fff7fu, y0 & 0xff80ff80u);
+    c23 = sub_bf16x2(y1 & 0xff7fff7fu, y1 & 0xff80ff80u);
+  }
+}
+// Entry v of the table: the byte selector (a dropped column takes a zero byte) and, above it,
+// the kept count.
+__device__ __forceinline__ uint32_t lut_entry(uint32_t v) {
+  uint32_t sel = 0, k = 0;
+  for (int j = 0; j < 4; ++j) sel |= ((v >> j & 1u) ? k++ : 4u) << (4 * j);
+  return sel | k << 16;
 }
 
 // 16 rows (two per lane) x 64 columns against NT token tiles.
 template <int ES, int NT, int S>
-__device__ __forceinline__ void tile_mma(uint32_t m0, uint32_t& pa0, uint32_t m1, uint32_t& pa1,
+__device__ __forceinline__ void tile_mma(uint32_t m0, uint32_t& pa0, uint32_t m1, uint32_t& pa1, uint32_t lut,
                                          const uint32_t (&xb)[NT][8], float (&acc)[NT][4]) {
-  const uint32_t a0 = expand2<ES, 2 * S>(m0, pa0);
-  const uint32_t a1 = expand2<ES, 2 * S>(m1, pa1);
-  const uint32_t a2 = expand2<ES, 2 * S + 1>(m0, pa0);
-  const uint32_t a3 = expand2<ES, 2 * S + 1>(m1, pa1);
+  uint32_t a0, a1, a2, a3;
+  expand4<ES, S>(m0, pa0, lut, a0, a2);
+  expand4<ES, S>(m1, pa1, lut, a1, a3);
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[nt], a0, a1, a2, a3, xb[nt][2 * S], xb[nt][2 * S + 1]);
-  if constexpr (S + 1 < 4) tile_mma<ES, NT, S + 1>(m0, pa0, m1, pa1, xb, acc);
+  if constexpr (S + 1 < 4) tile_mma<ES, NT, S + 1>(m0, pa0, m1, pa1, lut, xb, acc);
 }
 
 // y[m, n] from its FP32 sum v (INT8: times the row's scale sc) through the launch's epilogue
@@ -155,6 +179,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
     }
     fence_barrier_init();
   }
+  if (ES == 1 && warp == 1 && lane < 16) reinterpret_cast<uint32_t*>(smem + p.lut_off)[lane] = lut_entry(lane);
   __syncthreads();
   if (kPush && p.cluster > 1) cluster_arrive_relaxed();  // this CTA runs: its shared memory may be written
 
@@ -227,6 +252,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
   // a tile's loads are one 128-byte line, and the turn by q keeps the 16-byte stores of the scan,
   // in which lane l writes rows R l .. R l + R - 1, off each other's banks.
   uint32_t* tab = reinterpret_cast<uint32_t*>(smem + p.tab_off) + warp * RW * 4;
+  const uint32_t lut = smem_u32(smem + p.lut_off);
   const uint32_t tab_lane = smem_u32(tab) + 16u * g + 4u * t;
   const int turn = R == 4 ? (lane >> 1) & 3 : R == 2 ? (lane >> 2) & 1 : 0;
   float acc[kTiles][NT][4];
@@ -319,7 +345,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
         const uint32_t en0 = lds32((tab_lane ^ (16u * ((2 * i) % R))) + 256u * i);
         const uint32_t en1 = lds32((tab_lane ^ (16u * ((2 * i + 1) % R))) + 256u * i + 128u);
         uint32_t pa0 = vbase + (en0 >> 16) * ES, pa1 = vbase + (en1 >> 16) * ES;
-        tile_mma<ES, NT, 0>(en0, pa0, en1, pa1, xb, acc[i]);
+        tile_mma<ES, NT, 0>(en0, pa0, en1, pa1, lut, xb, acc[i]);
       }
     }
     __syncwarp();
@@ -414,7 +440,7 @@ struct MmaChoice {
 };
 struct MmaPlan {
   int slots, cluster;
-  uint32_t chunk_region, ring_off, tab_off, bar_off, rx_off;
+  uint32_t chunk_region, ring_off, tab_off, bar_off, lut_off, rx_off;
   size_t smem;
 };
 
@@ -491,7 +517,7 @@ bool mma_plan(const sp_matrix* h, int M, const MmaChoice& c, int occ, int min_sl
   const size_t tab = (size_t)c.cw * c.rw * 16;
   const int S = pl->cluster;
   const size_t rx = c.nt == 1 && c.cw == 8 && S > 1 ? (size_t)(M + S - 1) / S * S * kRows * sizeof(float) : 0;  // receive area
-  const size_t ctl = (size_t)kMaxSlots * (8 + 8 + 8 + 4) + rx;
+  const size_t ctl = (size_t)kMaxSlots * (8 + 8 + 8 + 4) + 64 + rx;  // barriers, tags, table, receive area
   const size_t per_slot = (size_t)c.nt * 1024 + pl->chunk_region;
   if (budget < tab + ctl + min_slots * per_slot) return false;
   const int items = (h->T + pl->cluster - 1) / pl->cluster;
@@ -502,6 +528,7 @@ bool mma_plan(const sp_matrix* h, int M, const MmaChoice& c, int occ, int min_sl
   const size_t ring_end = std::max<size_t>(pl->ring_off + (size_t)pl->slots * pl->chunk_region, (sums + 127) / 128 * 128);
   pl->tab_off = (uint32_t)ring_end;
   pl->bar_off = (uint32_t)(ring_end + tab);
+  pl->lut_off = (uint32_t)(pl->bar_off + kMaxSlots * (8 + 8 + 8 + 4));  // a multiple of 64
   pl->rx_off = (uint32_t)(pl->bar_off + ctl - rx);
   if (pl->bar_off + ctl > budget) return false;
   // The whole share of shared memory, whatever the chunks need: CTAs of consecutive launches
@@ -607,6 +634,7 @@ sp_status launch_linear_mma(const sp_matrix* h, const uint16_t* x, int64_t M, ui
   p.ring_off = pl.ring_off;
   p.tab_off = pl.tab_off;
   p.bar_off = pl.bar_off;
+  p.lut_off = pl.lut_off;
   p.rx_off = pl.rx_off;
   p.epi = epi;
   p.early = overlaps((int64_t)h->RB * pl.cluster, (int64_t)c.occ * h->num_sms) ? 1 : 0;
