@@ -510,13 +510,16 @@ size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
 // Against linear_tc_kernel, measured at 70 %: from 33 tokens on where the matrix is small or of
 // middling size (4096 x 4096 20 us against 33 at M = 64, 25 / 101 at 256; 1003 x 1096 10 / 63 at 64;
-// down 37 / 40 at 33, 53 / 111 at 256), later where the scratch is much traffic for few tokens
-// (q/k/v 39 / 36 at 64, 41 / 50 at 128; gate/up 79 / 59 at 128, 83 / 81 at 256, 94 / 120 at 384,
-// 218 / 376 at 2048).  A matrix of a few chunks keeps the one launch.
+// down, 5504 chunks, 37 / 40 at 33, 53 / 111 at 256), later where the scratch is much traffic for
+// few tokens (q/k/v, 6144 chunks, 41 / 36 at 64, 41 / 50 at 128; gate/up, 11008, 79 / 59 at 128,
+// 83 / 80 at 240, 94 / 120 at 384, 218 / 376 at 2048), and from ~250 tokens (INT8, which
+// linear_tc_kernel expands slower, ~200) whatever the size.  A matrix of a few chunks keeps the
+// one launch.
 bool uses_dense(const sp_matrix* h, int64_t M) {
   const int64_t C = (int64_t)h->RB * h->T, rows = (int64_t)h->RB * kRows;
   if (C < 16 || M > (int64_t)1 << 24 || (int64_t)h->T * rows >= (int64_t)1 << 31) return false;
-  return M > kMmaMaxRows && 24 * M >= C - 5000;
+  const int64_t from = h->esize == 2 ? std::min<int64_t>(250, (C - 5000) / 14) : std::min<int64_t>(200, (C - 5000) / 24);
+  return M > kMmaMaxRows && M >= from;
 }
 
 namespace {

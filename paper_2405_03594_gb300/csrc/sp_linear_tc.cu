@@ -31,7 +31,7 @@
 #include <cstring>
 #include <mutex>
 
-#include "sp_internal.cuh"
+#include "sp_expand.cuh"
 #include "sp_tcgen05.cuh"
 
 namespace sp {
@@ -56,58 +56,8 @@ constexpr size_t kSmemLimit = 226 * 1024;
 constexpr int kMaxDevices = 64;
 constexpr int kMaxSlots = 16;
 
-__device__ __forceinline__ uint16_t i8_to_bf16(uint32_t byte) {
-  const float f = __uint_as_float(0x4B000000u | (byte ^ 0x80u)) - 8388736.0f;
-  return (uint16_t)(__float_as_uint(f) >> 16);
-}
-
-// One output word (two adjacent columns) of a row's expansion, bf16 values: each kept
-// column takes the next value of the stream at shared address `pa` (which advances);
-// a dropped column gives +0.  Written in PTX so every column is one predicate-setting
-// AND, one predicated 16-bit shared load and one predicated pointer increment.
-template <uint32_t B0, uint32_t B1>
-__device__ __forceinline__ uint32_t expand_word_bf16(uint32_t m, uint32_t& pa) {
-  uint32_t o;
-  asm("{\n\t.reg .pred p0, p1;\n\t.reg .b32 t0, t1, lo, hi;\n\t"
-      "and.b32 t0, %2, %3;\n\t"
-      "setp.ne.b32 p0, t0, 0;\n\t"
-      "and.b32 t1, %2, %4;\n\t"
-      "setp.ne.b32 p1, t1, 0;\n\t"
-      "mov.b32 lo, 0;\n\t"
-      "mov.b32 hi, 0;\n\t"
-      "@p0 ld.shared.u16 lo, [%1];\n\t"
-      "@p0 add.u32 %1, %1, 2;\n\t"
-      "@p1 ld.shared.u16 hi, [%1];\n\t"
-      "@p1 add.u32 %1, %1, 2;\n\t"
-      "prmt.b32 %0, lo, hi, 0x5410;\n\t}"
-      : "=r"(o), "+r"(pa)
-      : "r"(m), "n"(B0), "n"(B1));
-  return o;
-}
-// The same for int8 values (one byte each), converted exactly to bf16.
-template <uint32_t B0, uint32_t B1>
-__device__ __forceinline__ uint32_t expand_word_i8(uint32_t m, uint32_t& pa) {
-  uint32_t lo = 0, hi = 0;
-  uint32_t b0, b1;
-  asm("{\n\t.reg .pred p0, p1;\n\t.reg .b32 t0, t1;\n\t"
-      "and.b32 t0, %3, %4;\n\t"
-      "setp.ne.b32 p0, t0, 0;\n\t"
-      "and.b32 t1, %3, %5;\n\t"
-      "setp.ne.b32 p1, t1, 0;\n\t"
-      "mov.b32 %0, 128;\n\t"
-      "mov.b32 %1, 128;\n\t"
-      "@p0 ld.shared.u8 %0, [%2];\n\t"
-      "@p0 add.u32 %2, %2, 1;\n\t"
-      "@p1 ld.shared.u8 %1, [%2];\n\t"
-      "@p1 add.u32 %2, %2, 1;\n\t}"
-      : "=r"(b0), "=r"(b1), "+r"(pa)
-      : "r"(m), "n"(B0), "n"(B1));
-  // a dropped column loads the byte 0x80 = -128 ... replaced below by +0
-  lo = (m & B0) ? i8_to_bf16(b0) : 0u;
-  hi = (m & B1) ? i8_to_bf16(b1) : 0u;
-  return lo | (hi << 16);
-}
-
+// Output words I and 16 + I (column pairs of the row's two halves), each half walking its own
+// value stream.  INT8: exact bf16 by one subtraction per pair.
 template <int ES, int I>
 __device__ __forceinline__ void expand_pair(uint32_t mlo, uint32_t mhi, uint32_t& pa, uint32_t& pb,
                                             uint32_t (&o)[32]) {
@@ -116,8 +66,8 @@ __device__ __forceinline__ void expand_pair(uint32_t mlo, uint32_t mhi, uint32_t
     o[I] = expand_word_bf16<B0, B1>(mlo, pa);
     o[16 + I] = expand_word_bf16<B0, B1>(mhi, pb);
   } else {
-    o[I] = expand_word_i8<B0, B1>(mlo, pa);
-    o[16 + I] = expand_word_i8<B0, B1>(mhi, pb);
+    o[I] = i8x2_to_bf16x2(expand_word_u8<B0, B1>(mlo, pa));
+    o[16 + I] = i8x2_to_bf16x2(expand_word_u8<B0, B1>(mhi, pb));
   }
   if constexpr (I + 1 < 16) expand_pair<ES, I + 1>(mlo, mhi, pa, pb, o);
 }
