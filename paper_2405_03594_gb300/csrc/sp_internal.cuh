@@ -76,7 +76,9 @@ struct LinearParams {
   uint64_t timeout_ns;
   int32_t cluster;      // CUDA-core kernel: > 1 = split each row block over this many CTAs of
                         // one thread-block cluster; <= 1 = stream-K over the workspace
-  uint32_t part_off;    // cluster mode: shared-memory offset of the CTA's FP32 partial
+  uint32_t part_off;    // cluster mode: shared-memory offset of the CTA's FP32 partial, or with
+  int32_t push;         // `push` of rank 0's receive area [cluster][kRows]: the other ranks store
+                        // their partials there instead of rank 0 reading theirs (one row)
   uint32_t comb_off;    // warp-per-chunk kernel: shared-memory offset of the warps' partials
   uint64_t probe_ns;    // 0, except in the failure-path test: consumer warp 0 of CTA 0 first
                         // waits this long on a barrier that nothing completes
