@@ -36,3 +36,21 @@ def test_integer_sums_bit_exact(oracle, N, K, M, int8):
         y = h.linear(gu.bf16_to_dev(x), path=path)
         sp.check()
         assert np.array_equal(gu.bf16_bits_from_dev(y), synth.bf16_from_f32(ref.astype(np.float32))), path
+
+
+@pytest.mark.parametrize("N,K", [(22016, 1152), (4096, 6400)])
+@pytest.mark.parametrize("M", [3, 16, 32])
+@pytest.mark.parametrize("least", [0.4, 1.0])
+def test_large_chunks_at_lower_occupancy(oracle, N, K, M, least):
+    """More than 20 chunks per SM whose size leaves fewer CTAs per SM than the kernel allows."""
+    from paper_2405_03594_gb300 import sp
+
+    g = np.random.default_rng(N + M)
+    mask = (g.random((N, K)) < g.uniform(least, 2 * least, size=(N, 1))).astype(np.uint8)
+    x = synth.bf16_from_f32(g.integers(-2, 3, size=(M, K)).astype(np.float32))
+    W = synth.bf16_from_f32(g.integers(-4, 5, size=(N, K)).astype(np.float32))
+    h = sp.compress(gu.bf16_to_dev(W), gu.u8_to_dev(mask))
+    y = h.linear(gu.bf16_to_dev(x))
+    sp.check()
+    ref = oracle.linear_bf16(x, W, mask)
+    assert np.array_equal(gu.bf16_bits_from_dev(y), synth.bf16_from_f32(ref.astype(np.float32)))
