@@ -29,10 +29,12 @@ bool live(const sp_matrix* h) { return h && h->magic == SP_MAGIC; }
 constexpr int64_t kCudaCoreMaxM_bf16 = 10;
 constexpr int64_t kCudaCoreMaxM_int8 = 13;
 
-// Workspace of the documented contract, whatever kernel runs a batch of m rows.
+// Workspace of the documented contract, whatever kernel runs a batch of m rows.  One size serves
+// every batch of more than 240 rows (the widest token tile), on either tensor-core route.
 size_t workspace_bytes(const sp_matrix* h, int64_t m) {
   const size_t b = std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m));
-  return uses_dense(h, m) ? std::max(b, workspace_bytes_dense(h, m)) : b;
+  const int64_t md = m > 240 ? 256 : m;
+  return uses_dense(h, md) ? std::max(b, workspace_bytes_dense(h, md)) : b;
 }
 
 bool uses_tensor_cores(const sp_matrix* h, int64_t m, sp_path path) {

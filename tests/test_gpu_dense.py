@@ -53,6 +53,20 @@ def test_integer_sums_bit_exact(oracle, N, K, M, int8):
     assert np.array_equal(gu.bf16_bits_from_dev(y)[:, rows], synth.bf16_from_f32(ref.astype(np.float32)))
 
 
+@pytest.mark.parametrize("int8", [False, True])
+@pytest.mark.parametrize("N,K", [(8960, 8192), (2048, 1024)])
+def test_one_workspace_size_above_240_rows(N, K, int8):
+    """A workspace sized for one batch of more than 240 rows serves every other one, and none
+    of fewer rows needs more."""
+    from paper_2405_03594_gb300 import sp
+
+    g = np.random.default_rng(9)
+    _, h = _matrix(sp, N, K, int8, g)
+    size = h.workspace_size(241)
+    assert {h.workspace_size(m) for m in (249, 250, 256, 2048, (1 << 24) + 1)} == {size}
+    assert max(h.workspace_size(m) for m in (1, 2, 16, 32, 33, 100, 200, 240)) <= size
+
+
 def test_update_then_large_batch_on_one_stream(oracle):
     """The expansion reads the values that a masked update before it on the stream wrote."""
     from paper_2405_03594_gb300 import sp
