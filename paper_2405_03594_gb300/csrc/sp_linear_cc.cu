@@ -958,9 +958,9 @@ sp_status launch_linear_cc(const sp_matrix* h, const uint16_t* x, int64_t M, uin
   // the configuration depends on the batch rows of a launch: full launches of kMaxTokens
   // rows and one ragged tail; the workspace is checked before the first launch
   const bool probe = probe_ns != 0;
-  // Most batches of more than one row run on linear_mma_kernel, which needs no workspace, except
-  // where the caller wants this file's kernels: the no-allocation entry point and the
-  // failure-path test.
+  // Most batches of more than one row, and one row of an INT8 matrix that keeps many weights, run
+  // on linear_mma_kernel, which needs no workspace, except where the caller wants this file's
+  // kernels: the no-allocation entry point and the failure-path test.
   auto on_mma = [&](int Mt) { return allow_cluster && !probe && uses_mma(h, Mt); };
   auto stream_k = [&](int Mt) {
     CcPlan q;

@@ -628,10 +628,19 @@ sp_status dispatch(const sp_matrix* h, const MmaParams& p, const CUtensorMap& ma
 
 }  // namespace
 
-// Two rows of a large matrix stay with the kept-weight walk (M = 2, 80 %: down 15.0 us against
-// 17.1 here; INT8 at 70 % 20.2 / 21.9; the other shapes within a few percent of each other).
+// One row, and two of a large matrix, stay with the kept-weight walk, whose time follows the
+// weights kept, except where an INT8 matrix keeps many: its walk takes an instruction more per
+// weight, the expansion here the same time at any sparsity.  Four layers of the Llama-2 7B stack,
+// INT8, walk / here: M = 2 at 50 % 592 / 334 us, 60 % 396 / 334, 70 % 350 / 332, 80 % 299 / 331;
+// M = 1 (the o linear, 14 chunks per SM, on the walk) at 50 % 383 / 321, at 60 % 341 / 321, at 70 %
+// 299 / 321.  bf16 at M = 2: 364 / 370, 327 / 350, 295 / 319, 260 / 294; at M = 1 357 / 389,
+// 307 / 359, 263 / 321, 224 / 298.
 bool uses_mma(const sp_matrix* h, int64_t M) {
-  if (M < 2 || M > kMmaMaxRows || (M == 2 && large(h))) return false;
+  if (M < 1 || M > kMmaMaxRows || (M == 1 && !large(h))) return false;
+  if (M == 1 || (M == 2 && large(h))) {
+    const double kept = (double)h->nnz / ((double)h->N * (double)h->K);
+    if (h->esize == 2 || kept < (M == 1 ? 0.36 : 0.26)) return false;
+  }
   MmaChoice c;
   MmaPlan pl;
   return choose(h, (int)M, &c, &pl);

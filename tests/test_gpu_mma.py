@@ -54,3 +54,31 @@ def test_large_chunks_at_lower_occupancy(oracle, N, K, M, least):
     sp.check()
     ref = oracle.linear_bf16(x, W, mask)
     assert np.array_equal(gu.bf16_bits_from_dev(y), synth.bf16_from_f32(ref.astype(np.float32)))
+
+
+@pytest.mark.parametrize("N,K", [(22016, 1152), (4096, 6408)])
+@pytest.mark.parametrize("keep", [0.30, 0.36, 0.5, 1.0])  # either side of the lines at 0.36 and 0.26
+@pytest.mark.parametrize("M", [1, 2])
+def test_one_and_two_rows_of_many_int8_weights(oracle, N, K, keep, M):
+    """INT8 matrices that keep many weights: the products and the residual epilogue."""
+    import torch
+
+    from paper_2405_03594_gb300 import sp
+
+    g = np.random.default_rng(N + M)
+    mask = (g.random((N, K)) < keep).astype(np.uint8)
+    q = g.integers(-128, 128, size=(N, K)).astype(np.int8)
+    s = np.exp2(g.integers(-3, 4, size=N)).astype(np.float32)
+    x = synth.bf16_from_f32(g.integers(-2, 3, size=(M, K)).astype(np.float32))
+    h = sp.compress(gu.i8_to_dev(q), gu.u8_to_dev(mask), gu.f32_to_dev(s))
+    ws = torch.zeros(max(h.workspace_size(M), 256), dtype=torch.uint8, device=gu.dev())
+    y = h.linear(gu.bf16_to_dev(x), workspace=ws)
+    ref = oracle.linear_int8(x, q, mask, s)
+    assert np.array_equal(gu.bf16_bits_from_dev(y), synth.bf16_from_f32(ref.astype(np.float32)))
+    h0 = gu.bf16_to_dev(synth.activations(M, N, g))
+    r = gu.bf16_to_dev(synth.activations(1, N, g)[0])
+    h1 = h0.clone()
+    assert h.linear_epi(gu.bf16_to_dev(x), h1, "residual", r, workspace=ws)
+    sp.residual_add(h0, y, r)
+    sp.check()
+    assert np.array_equal(gu.bf16_bits_from_dev(h1), gu.bf16_bits_from_dev(h0))
