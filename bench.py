@@ -373,7 +373,7 @@ def dense_section(host, xs, results, Ms):
 KERNEL_SOURCES = {
     "linear_ccw_kernel": ("sp_linear_cc.cu", "sp_cc_common.cuh", "sp_internal.cuh"),
     "linear_cc_kernel": ("sp_linear_cc.cu", "sp_cc_common.cuh", "sp_internal.cuh"),
-    "linear_tc_kernel": ("sp_linear_tc.cu", "sp_internal.cuh"),
+    "linear_tc_kernel": ("sp_linear_tc.cu", "sp_expand.cuh", "sp_tcgen05.cuh", "sp_internal.cuh"),
     "chain_kernel": ("sp_chain.cu", "sp_cc_common.cuh", "sp_internal.cuh"),
 }
 

@@ -67,8 +67,8 @@ typedef enum sp_dtype { SP_BF16 = 0, SP_INT8 = 1 } sp_dtype;
    family for M <= 10 (bf16 values) or M <= 13 (int8 values), the tensor-core family above. */
 typedef enum sp_path {
   SP_PATH_AUTO = 0,
-  SP_PATH_CUDA_CORE = 1,    /* popc-prefix expansion, FP32 FMA on CUDA cores */
-  SP_PATH_TENSOR_CORE = 2   /* expansion into tensor memory, tcgen05 MMA */
+  SP_PATH_CUDA_CORE = 1,    /* FP32 FMA over the kept weights; from 2 rows mostly warp-level MMA */
+  SP_PATH_TENSOR_CORE = 2   /* warp-level MMA up to 32 rows; tcgen05 MMA above */
 } sp_path;
 
 typedef struct sp_matrix sp_matrix; /* opaque; owns the compressed weight */
@@ -134,14 +134,14 @@ sp_status sp_linear_ex(const sp_matrix* h, const void* x_dev, int64_t m, void* y
                        size_t workspace_bytes, sp_path path, void* stream);
 
 /* Kernels that sp_linear_ex can launch (reported by sp_launch_count): the family's choice for
-   the batch.  Within either family, batches of 2 .. 32 rows mostly run on linear_mma_kernel
+   the batch.  Within either family, batches of up to 32 rows mostly run on linear_mma_kernel
    (warp-level matrix instructions on chunks expanded in registers), which is the faster one
    there; the report stays the family's. */
 enum {
   SP_KERNEL_NONE = 0,
   SP_KERNEL_CC_THREAD_PER_ROW = 1,  /* linear_cc_kernel: four warps share a chunk, thread = row */
   SP_KERNEL_CC_WARP_PER_CHUNK = 2,  /* linear_ccw_kernel (M <= 4): a warp per chunk, lane = 4 rows */
-  SP_KERNEL_TENSOR_CORE = 3         /* linear_tc_kernel */
+  SP_KERNEL_TENSOR_CORE = 3         /* linear_tc_kernel; expand_kernel and dense_kernel for 2 launches */
 };
 
 /* (Library plumbing; no counterpart in the paper.)  Number of kernel launches that
@@ -216,16 +216,16 @@ sp_status sp_linear_w8a8(const sp_matrix* h, const int8_t* qx_dev, const float* 
 sp_status sp_w8a8_workspace_size(const sp_matrix* h, int64_t m, size_t* bytes);
 
 /* Failure-path test (the paper has no counterpart; nothing calls it in normal use).  Runs
- * sp_linear's CUDA-core decode kernel for m = 1..4 rows -- the warp-per-chunk kernel, as
- * sp_linear would -- with one consumer warp of its first CTA first waiting on a
+ * the CUDA-core decode kernel for m = 1..4 rows -- the warp-per-chunk kernel -- with one
+ * consumer warp of its first CTA first waiting on a
  * shared-memory barrier that nothing completes and no copy targets.  That bounded wait gives
  * up after wait_ms milliseconds and records SP_ERR_TIMEOUT in the device status word, as any
  * expired wait does; the warp then goes on normally, so the launch ends and y is the product
  * sp_linear would give.  Afterwards sp_check() returns SP_ERR_TIMEOUT once (and clears the
  * status), and the workspace is ready for the next call.  Arguments as for sp_linear;
  * wait_ms in 1..10000 (SP_ERR_INVALID_ARG otherwise); SP_ERR_UNSUPPORTED when m is outside
- * 1..4, for an SP_INT8 handle, or when sp_linear would not run the warp-per-chunk kernel
- * for this matrix.  The waiting warp is compiled into a variant of the kernel of its own;
+ * 1..4, for an SP_INT8 handle, or when the warp-per-chunk kernel does not fit this matrix
+ * and batch.  The waiting warp is compiled into a variant of the kernel of its own;
  * sp_linear never runs that variant. */
 sp_status sp_test_expired_wait(const sp_matrix* h, const void* x_dev, int64_t m, void* y_dev, void* workspace_dev,
                                size_t workspace_bytes, uint32_t wait_ms, void* stream);

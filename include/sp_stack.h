@@ -101,8 +101,8 @@ sp_status sp_chain_run(const sp_chain_op* ops, int32_t n_ops, int64_t m, void* w
  * sp_mul_pairs (bitwise, for the same kernel and batch).  x [m, K] and y are bf16,
  * contiguous and 16-byte aligned; r is bf16 [N] for SP_EPI_RESIDUAL, else NULL; the
  * workspace is as for sp_linear (sp_workspace_size bytes, zero-filled once, calls that
- * share it ordered on one stream).  Runs on the CUDA-core kernels: where the automatic path
- * takes the tensor-core kernel for m rows the call returns SP_ERR_UNSUPPORTED without a
+ * share it ordered on one stream).  Runs on the CUDA-core family: where the automatic path
+ * takes the tensor-core family for m rows the call returns SP_ERR_UNSUPPORTED without a
  * launch, and the caller uses sp_linear and the glue call instead.  Other errors as
  * sp_linear, and SP_ERR_INVALID_ARG for an unknown epilogue, a missing r or an odd N with
  * the pair product. */

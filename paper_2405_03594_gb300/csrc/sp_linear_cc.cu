@@ -5,8 +5,9 @@
 // memory onto the chip and are expanded there by their bitmask; decode is bound
 // by those bytes, Sec. 2.4, 3.4).
 //
-// sp_linear runs these kernels for one row, and for two rows of a large matrix; other batches
-// of up to 32 rows go to linear_mma_kernel (sp_linear_mma.cu).  More rows run here for the
+// sp_linear runs these kernels for one row, and for two rows of a large matrix, unless it is an
+// INT8 matrix that keeps many weights; other batches of up to 32 rows go to linear_mma_kernel
+// (uses_mma, sp_linear_mma.cu).  More rows run here for the
 // no-allocation entry point and the failure-path test.
 //
 // Launch: each row block split over the S CTAs of a thread-block cluster (up to two rows;

@@ -1,12 +1,12 @@
-// sp_linear_mma.cu -- sparse linear for batches of 2 .. 32 rows: chunks expanded in
-// registers straight into the operands of warp-level matrix instructions.
+// sp_linear_mma.cu -- sparse linear for batches of 2 .. 32 rows, and for one row of an INT8
+// matrix that keeps many weights: chunks expanded in registers straight into the operands of
+// warp-level matrix instructions.
 //
 // Between one row (linear_ccw_kernel walks the kept weights only) and a few dozen rows the
 // product is bound by neither HBM nor the tensor pipe but by the work of turning a chunk's
 // mask and packed values into operands.  A walk over kept weights on the CUDA cores pays M
-// multiply-adds and M / 2 shuffles per weight; the tcgen05 kernel pays ~250 ns per chunk on
-// its issuing thread (a tcgen05.mma costs ~80 cycles to issue however few tokens it has)
-// plus the trip through tensor memory.  Here a warp expands 16 columns of two rows per lane
+// multiply-adds and M / 2 shuffles per weight; the tcgen05 kernel pays the trip through tensor
+// memory on one CTA per SM, whatever the tokens.  Here a warp expands 16 columns of two rows per lane
 // directly into the A registers of mma.sync m16n8k16 (bf16, FP32 accumulation), so the cost
 // of a chunk hardly depends on M: four matrix instructions per 16 rows and 8 tokens beside
 // ~290 instructions of expansion.  What bounds it is shared memory: ~530 wavefronts per chunk
@@ -14,7 +14,7 @@
 // (ncu), the rest being launch latency and tail.  Measured at 70 %, bf16, graphs of launches on
 // matrices beyond L2, before / here: gate/up 32.2 / 28.1 us at M = 3, 48.7 / 28.4 at M = 5,
 // 61.6 / 31.5 at M = 10, 46.4 / 32.1 at M = 16, 47.2 / 40.9 at M = 32; o 15.3 / 8.8, 18.2 / 9.6,
-// 20.9 / 9.8, 23.4 / 12.8 at M = 5, 10, 16, 32; INT8 gate/up 54 / 34.6 at M = 5, 55.5 / 40.0 at
+// 20.9 / 9.8, 23.4 / 12.8 at M = 5, 10, 16, 32; INT8 gate/up 54 / 30.8 at M = 5, 55.5 / 35.0 at
 // M = 16.
 //
 // The product is free to permute K: in k-step s, lane (g, t) of a warp (g = lane / 4,
@@ -27,13 +27,14 @@
 //                    x 64 columns, 128-byte swizzle; tokens past M and columns past K read as
 //                    zero) into a ring of `slots` slots, full/empty mbarriers.
 //   warps 0..CW-1    consumers.  128 / RW warps share a chunk, each taking RW of its rows; the
-//                    CTA has CW * RW / 128 chunks in work.  A warp scans the popcounts of its 16-column mask pieces into a table
-//                    (mask piece, first value) of its own, and expands and multiplies 16 rows
-//                    at a time.
+//                    CTA has CW * RW / 128 chunks in work.  A warp scans the popcounts of its
+//                    16-column mask pieces into a table (mask piece, first value) of its own,
+//                    and expands and multiplies 16 rows at a time.
 // At the end of its K-tiles a CTA adds its warps' sums in warp order in shared memory (on the
 // ring, which is idle by then); the cluster's CTAs then each sum a share of the tokens over
 // all ranks in rank order (distributed shared memory: pushed to the owner by the eight-warp form
-// up to 8 tokens, read by it otherwise) and write y through the launch's output epilogue.  All orders are fixed: results are bitwise repeatable.
+// up to 8 tokens, read by it otherwise) and write y through the launch's output epilogue.  All
+// orders are fixed: results are bitwise repeatable.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

@@ -2,8 +2,10 @@
 //
 // The GPU engine of Sec. 2.4.2: compressed submatrices move from global memory onto
 // the chip, are expanded by their bitmask, and the tensor cores run on the expanded
-// tiles at the dense rate while global traffic stays at the compressed size.  On
-// sm_103a the expanded tile goes to tensor memory and feeds tcgen05.mma directly:
+// tiles at the dense rate while global traffic stays at the compressed size.  This kernel
+// takes the batches of more than 32 rows (below, linear_mma_kernel) that do not repay
+// expanding the whole matrix first (uses_dense).  On sm_103a the expanded tile goes to tensor
+// memory and feeds tcgen05.mma directly:
 //
 //   D[128 rows, Ntok tokens] (fp32, TMEM) += A[128 rows, 64 k] (bf16, TMEM) x B[64 k, Ntok]
 //
@@ -14,7 +16,7 @@
 //   warp 0 lane 0   producer: cp.async.bulk of each chunk and a TMA tile of x into a
 //                   ring of S shared-memory slots; item n uses slot n % S and TMEM A
 //                   stage n % S, and one MMA commit frees both (stage_free[n % S]);
-//   warp 1          TMEM allocation; lane 0 issues the MMAs (4 x K=16 per chunk) and
+//   warp 1          TMEM allocation; one elected lane issues the MMAs (4 x K=16 per chunk) and
 //                   commits them to mbarriers that free the stage and, at a segment's
 //                   end, hand D to the epilogue;
 //   warps 2-..      EG expander warpgroups taking chunks round-robin: thread r of a
