@@ -130,6 +130,35 @@ __device__ __forceinline__ void store_y_block(const TcParams& tp, const CUtensor
   }
 }
 
+// The sum of segment sg's partials, all read from memory in CTA order; returns the next staging
+// buffer.  Not inlined: rare, and its registers would spill in the expanders' loop.
+__device__ __noinline__ int sum_partials(const TcParams& tp, const CUtensorMap* tmap_y, uint16_t* stg, int step,
+                                         int64_t sg, float sc, int r, int tid128, int bar) {
+  const LinearParams& p = tp.p;
+  const int part = kRows * tp.ntok;
+  const int64_t seg_begin = sg * p.T;
+  const int first = (int)owner_of(seg_begin, p.W, p.G), last = (int)owner_of(seg_begin + p.T - 1, p.W, p.G);
+  const int sf = (range_begin(first, p.W, p.G) / p.T == sg) ? 0 : 1;
+  for (int c0 = 0; c0 < tp.ntok; c0 += 32) {
+    float sum[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) sum[i] = 0.f;
+    const int nv = tp.ntok - c0 < 32 ? tp.ntok - c0 : 32;
+    for (int ci = first; ci <= last; ++ci) {
+      // the segment is the first of every CTA but the first
+      const float* src = p.ws + (int64_t)(ci * 2 + (ci == first ? sf : 0)) * part + c0 * kRows + r;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) sum[i] += __ldcg(src + i * kRows);
+      if (nv == 32) {
+#pragma unroll
+        for (int i = 16; i < 32; ++i) sum[i] += __ldcg(src + i * kRows);
+      }
+    }
+    store_y_block(tp, tmap_y, stg, step, sum, sc, nv, sg / p.RB * tp.ntok + c0, sg % p.RB, r, tid128, bar);
+  }
+  return step;
+}
+
 // TMEM split for a token tile of ntok columns: D buffers first, A stages after.  Small
 // tiles (decode) leave room for two D buffers and up to 14 A stages, so neither the
 // epilogue of one (row block, token tile) segment nor the tcgen05.commit round trip that
@@ -406,22 +435,26 @@ __global__ void __launch_bounds__(tc_threads(EG), 1)
       // segment ends early in the launch, its last one at the end, so at the end they mostly
       // have.  This CTA then adds theirs to its own sums straight from TMEM (the same sum as
       // below, in CTA order, as long as at most one CTA comes before it).
-      // Writing its own sums to memory, fencing and reading them all back took the launch's last
-      // 5 to 20 us: gate/up, 70 %, 46.2 -> 41.7 us at M = 64, 59.4 -> 48.9 at 128, 79.0 -> 60.0
-      // at 240; INT8 53.5 -> 48.4 and 68.1 -> 56.5 at 64 and 128.
-      // others: 0 if not, else 1 + 2 (slot of the partial of the CTA before) + 4 (there is one)
-      // + 8 (CTAs after).
+      // Otherwise it leaves its own and counts; if that makes it the last one and D is not
+      // needed for another segment, it does the same then.
+      // others: 0 while partials are missing, else 1 + 2 (slot of the first CTA's partial) +
+      // 4 (CTAs before) + 4096 (CTAs after); -1 if all partials are to be read from memory.
+      // Reading them all back, its own too, took the launch's last 5 to 20 us: gate/up, 70 %,
+      // 46.2 -> 41.8 us at M = 64, 59.4 -> 49.0 at 128, 79.0 -> 60.3 at 240, INT8 53.5 -> 49.1
+      // and 68.1 -> 56.8 at 64 and 128; q/k/v, most of whose row blocks are shared by CTAs that
+      // end together, 36.0 -> 31.6 at 64, 42.7 -> 33.2 at 80.
       int others = 0;
       if (!complete) {
         if (tid128 == 0) {
-          const int me = (int)blockIdx.x;
-          const int first = (int)owner_of(seg_begin, p.W, p.G);
-          const int n = (int)owner_of(seg_begin + T - 1, p.W, p.G) - first;
-          const int sf = (range_begin(first, p.W, p.G) / T == sg) ? 0 : 1;
-          int* ctr = p.cnt + first * 2 + sf;
-          const bool all = me - first <= 1 && ld_acquire_gpu(ctr) == n;
+          const int before = (int)blockIdx.x - (int)owner_of(seg_begin, p.W, p.G);
+          const int after = (int)owner_of(seg_begin + T - 1, p.W, p.G) - (int)blockIdx.x;
+          const int sf = (range_begin(blockIdx.x - before, p.W, p.G) / T == sg) ? 0 : 1;
+          const int code = 1 + 2 * sf + 4 * before + 4096 * after;
+          s_flag[kMaxExpGroups + grp] = code;
+          int* ctr = p.cnt + ((int)blockIdx.x - before) * 2 + sf;
+          const bool all = before <= 1 && ld_acquire_gpu(ctr) == before + after;
           if (all) atomicExch(ctr, 0);
-          s_flag[grp] = all ? 1 + 2 * sf + 4 * (me - first) + 8 * (n - (me - first)) : 0;
+          s_flag[grp] = all ? code : 0;
         }
         named_bar_sync(bar, 128);
         others = s_flag[grp];
@@ -436,77 +469,71 @@ __global__ void __launch_bounds__(tc_threads(EG), 1)
       tc_fence_after();
       const int my_slot = (sg == sg_first) ? 0 : 1;
       const int part = kRows * tp.ntok;  // floats per partial slot
-      for (int c0 = 0; c0 < tp.ntok; c0 += 32) {
-        uint32_t v[32];
-        if (!dead) {
-          tmem_load32(d_taddr + lane_base + (uint32_t)c0, v);
-          tmem_load_wait();
-        }
-        const int nv = tp.ntok - c0 < 32 ? tp.ntok - c0 : 32;  // ntok is a multiple of 16
-        if (complete || others) {
-          const float zero = others ? 0.f : -0.f;  // the sum below starts from 0
-          float a[32];
-#pragma unroll
-          for (int i = 0; i < 32; ++i) a[i] = zero + __uint_as_float(v[i]);
 #pragma unroll 1
-          for (int j = -((others >> 2) & 1); j <= others >> 3; ++j) {
-            if (j == 0) continue;
-            // a CTA after this one has the segment as its first
-            const int sl = j < 0 ? (others >> 1) & 1 : 0;
-            const float* src = p.ws + (int64_t)((int)(blockIdx.x + j) * 2 + sl) * part + c0 * kRows + r;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) a[i] += __ldcg(src + i * kRows);
-            if (nv == 32) {
-#pragma unroll
-              for (int i = 16; i < 32; ++i) a[i] += __ldcg(src + i * kRows);
-            }
+      for (;;) {
+        for (int c0 = 0; c0 < tp.ntok; c0 += 32) {
+          uint32_t v[32];
+          if (!dead) {
+            tmem_load32(d_taddr + lane_base + (uint32_t)c0, v);
+            tmem_load_wait();
           }
-          store_y_block(tp, &tmap_y, stg, stg_step, a, sc, nv, mtile * tp.ntok + c0, rb, r, tid128, bar);
-        } else {
-          float* wsp = p.ws + (int64_t)((int)blockIdx.x * 2 + my_slot) * part + c0 * kRows + r;
+          const int nv = tp.ntok - c0 < 32 ? tp.ntok - c0 : 32;  // ntok is a multiple of 16
+          if (complete || others) {
+            const float zero = others ? 0.f : -0.f;  // the sum below starts from 0
+            float a[32];
 #pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (i < nv) __stcg(wsp + i * kRows, __uint_as_float(v[i]));
+            for (int i = 0; i < 32; ++i) a[i] = zero + __uint_as_float(v[i]);
+#pragma unroll 1
+            for (int j = -((others >> 2) & 1); j <= others >> 12; ++j) {
+              if (j == 0) continue;
+              // a CTA after this one has the segment as its first
+              const int sl = j < 0 ? (others >> 1) & 1 : 0;
+              const float* src = p.ws + (int64_t)((int)(blockIdx.x + j) * 2 + sl) * part + c0 * kRows + r;
+#pragma unroll
+              for (int i = 0; i < 16; ++i) a[i] += __ldcg(src + i * kRows);
+              if (nv == 32) {
+#pragma unroll
+                for (int i = 16; i < 32; ++i) a[i] += __ldcg(src + i * kRows);
+              }
+            }
+            store_y_block(tp, &tmap_y, stg, stg_step, a, sc, nv, mtile * tp.ntok + c0, rb, r, tid128, bar);
+          } else {
+            float* wsp = p.ws + (int64_t)((int)blockIdx.x * 2 + my_slot) * part + c0 * kRows + r;
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              if (i < nv) __stcg(wsp + i * kRows, __uint_as_float(v[i]));
+          }
         }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&d_empty[db]);
-      if (others) {
-        named_bar_sync(bar, 128);  // every thread has read s_flag
-      } else if (!complete) {
+        if (complete || others > 0) break;
+        // D is free for the next segment, unless this is the CTA's last
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&d_empty[db]);
         __threadfence();
         named_bar_sync(bar, 128);
-        const int64_t i_first = owner_of(seg_begin, p.W, p.G);
-        const int64_t i_last = owner_of(seg_begin + T - 1, p.W, p.G);
-        const int sf = (range_begin(i_first, p.W, p.G) / T == sg) ? 0 : 1;
-        int* ctr = p.cnt + i_first * 2 + sf;
         if (tid128 == 0) {
-          const int old = atomicAdd(ctr, 1);
-          s_flag[grp] = (old == (int)(i_last - i_first)) ? 1 : 0;
-        }
-        named_bar_sync(bar, 128);
-        if (s_flag[grp]) {
-          __threadfence();
-          // 32 tokens at a time: each contributor's 32 partials are independent loads
-          for (int c0 = 0; c0 < tp.ntok; c0 += 32) {
-            float sum[32];
-#pragma unroll
-            for (int i = 0; i < 32; ++i) sum[i] = 0.f;
-            for (int64_t ci = i_first; ci <= i_last; ++ci) {
-              const int sl = (range_begin(ci, p.W, p.G) / T == sg) ? 0 : 1;
-              const float* src = p.ws + (ci * 2 + sl) * part + c0 * kRows + r;
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                if (c0 + i < tp.ntok) sum[i] += __ldcg(src + (int64_t)i * kRows);
-            }
-            const int nv = tp.ntok - c0 < 32 ? tp.ntok - c0 : 32;
-            store_y_block(tp, &tmap_y, stg, stg_step, sum, sc, nv, mtile * tp.ntok + c0, rb, r, tid128, bar);
+          const int code = s_flag[kMaxExpGroups + grp], before = (code >> 2) & 1023, after = code >> 12;
+          int* ctr = p.cnt + ((int)blockIdx.x - before) * 2 + ((code >> 1) & 1);
+          int f = 0;
+          if (atomicAdd(ctr, 1) == before + after) {
+            __threadfence();
+            atomicExch(ctr, 0);
+            f = before <= 1 && w + 1 == w1 ? code : -1;
           }
-          if (tid128 == 0) atomicExch(ctr, 0);
+          s_flag[grp] = f;
         }
         named_bar_sync(bar, 128);
+        others = s_flag[grp];
+        if (others <= 0) break;  // else: once more, with D still in place
       }
+      if (complete || (others > 0)) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&d_empty[db]);
+      }
+      if (others < 0)
+        stg_step = sum_partials(tp, &tmap_y, stg, stg_step, sg, sc, r, tid128, bar);
+      if (!complete) named_bar_sync(bar, 128);  // every thread has read s_flag
     }
   }
   if (tp.y_tma && warp >= kExpWarp0 && ((warp - kExpWarp0) & 3) == 0 && lane == 0) bulk_wait_all();
