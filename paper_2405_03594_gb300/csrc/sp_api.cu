@@ -33,7 +33,7 @@ constexpr int64_t kCudaCoreMaxM_int8 = 13;
 // every batch of more than 240 rows (the widest token tile), on either tensor-core route.
 size_t workspace_bytes(const sp_matrix* h, int64_t m) {
   const size_t b = std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m));
-  const int64_t md = m > 240 ? 256 : m;
+  const int64_t md = m > 240 ? 257 : m;  // as uses_dense has it from there on
   return uses_dense(h, md) ? std::max(b, workspace_bytes_dense(h, md)) : b;
 }
 

@@ -508,17 +508,18 @@ size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
 }  // namespace
 
-// Against linear_tc_kernel, measured at 70 %: from 33 tokens on where the matrix is small or of
-// middling size (4096 x 4096 20 us against 33 at M = 64, 25 / 101 at 256; 1003 x 1096 10 / 63 at 64;
-// down, 5504 chunks, 37 / 40 at 33, 53 / 111 at 256), later where the scratch is much traffic for
-// few tokens (q/k/v, 6144 chunks, 41 / 36 at 64, 41 / 50 at 128; gate/up, 11008, 79 / 59 at 128,
-// 83 / 80 at 240, 94 / 120 at 384, 218 / 376 at 2048), and from ~250 tokens (INT8, which
-// linear_tc_kernel expands slower, ~200) whatever the size.  A matrix of a few chunks keeps the
-// one launch.
+// Against linear_tc_kernel (one token tile up to 256 rows), measured at 70 %, this way / that, us.
+// bf16: small matrices from 33 tokens on (o, 2048 chunks, 19.5 / 24.7 at 33, 25.0 / 51.9 at 256);
+// middling ones from ~110 (8192 x 4096, 28.8 / 28.1 at 80, 32.4 / 36.7 at 160; down, 5504 chunks,
+// 39.7 / 36.1 and 45.0 / 47.2); where the scratch is much traffic for few tokens only beyond one
+// token tile (q/k/v, 6144 chunks, 41.3 / 31.8 at 64, 49.8 / 48.5 at 256; gate/up, 11008, 76.5 / 42.0
+// and 82.4 / 61.9; two tiles 94 / 120 at 384).  INT8, which linear_tc_kernel expands slower: down
+// 37.5 / 39.7 at 64, q/k/v 41.9 / 41.7 at 128, 14336 x 4096 (7168 chunks) 51.4 / 50.8 at 192, gate/up
+// 82.9 / 67.5 at 256.  A matrix of a few chunks keeps the one launch.
 bool uses_dense(const sp_matrix* h, int64_t M) {
   const int64_t C = (int64_t)h->RB * h->T, rows = (int64_t)h->RB * kRows;
   if (C < 16 || M > (int64_t)1 << 24 || (int64_t)h->T * rows >= (int64_t)1 << 31) return false;
-  const int64_t from = h->esize == 2 ? std::min<int64_t>(250, (C - 5000) / 14) : std::min<int64_t>(200, (C - 5000) / 24);
+  const int64_t from = h->esize == 2 ? (C < 4000 ? 33 : C < 6000 ? 110 : 257) : std::min<int64_t>(257, (C - 5400) / 10 + 33);
   return M > kMmaMaxRows && M >= from;
 }
 

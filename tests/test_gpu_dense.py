@@ -63,7 +63,7 @@ def test_one_workspace_size_above_240_rows(N, K, int8):
     g = np.random.default_rng(9)
     _, h = _matrix(sp, N, K, int8, g)
     size = h.workspace_size(241)
-    assert {h.workspace_size(m) for m in (249, 250, 256, 2048, (1 << 24) + 1)} == {size}
+    assert {h.workspace_size(m) for m in (249, 250, 256, 257, 2048, (1 << 24) + 1)} == {size}
     assert max(h.workspace_size(m) for m in (1, 2, 16, 32, 33, 100, 200, 240)) <= size
 
 
