@@ -164,6 +164,21 @@ __device__ __forceinline__ bool mbar_wait_sleep(uint64_t* bar, uint32_t parity, 
     if (global_ns() - t0 > timeout_ns) return false;
   }
 }
+// Bounded wait until a ring slot's tag names item n, for consumers that share the ring without
+// reading every item: the slot may still hold an earlier item of another warp, and the producer
+// claims it for n only once that one was consumed, so a parity wait that follows the claim cannot
+// match an older phase of the slot's barrier.  The tag changes while the lanes look at it, so
+// they may leave at different times: no vote or shuffle in here, and none under a condition on a
+// tag elsewhere.  The caller votes once, over this wait and the barrier's, where all lanes are.
+__device__ __forceinline__ bool wait_claimed(const volatile int* tag, int n, uint64_t timeout_ns) {
+  if (*tag == n) return true;
+  const uint64_t t0 = global_ns();
+  do {
+    __nanosleep(32);
+    if (*tag == n) return true;
+  } while (global_ns() - t0 <= timeout_ns);
+  return false;
+}
 // 1-D bulk copy global -> shared, completing `bytes` of transaction on `bar`.
 // dst, src and bytes must be multiples of 16.
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {

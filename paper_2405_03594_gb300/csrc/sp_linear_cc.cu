@@ -655,27 +655,12 @@ __global__ void __launch_bounds__(kThreads, OCC) linear_ccw_kernel(const LinearP
 #pragma unroll
       for (int m = 0; m < M; ++m) acc[i][m] = 0.f;
     for (; w < we; w += kConsumerWarps) {
-      if (!dead && tag[s] != (int)(w - w0)) {
-        // the slot may still hold an earlier item of another warp: wait until the producer
-        // has claimed it for this one (it does so only once that item was consumed), so
-        // the parity wait below cannot match an older phase of the slot's barrier
-        const uint64_t t0 = global_ns();
-        while (tag[s] != (int)(w - w0)) {
-          __nanosleep(32);
-          if (global_ns() - t0 > p.timeout_ns) {
-            dead = true;
-            set_status(p.status, kStatusTimeout);
-            break;
-          }
-        }
-        dead = __any_sync(0xffffffffu, dead);
-      }
-      if (!dead) {
-        const bool ok = __all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.timeout_ns));
-        if (!ok) {
-          dead = true;
-          set_status(p.status, kStatusTimeout);
-        }
+      // one vote, in front of which every lane comes: the slot is claimed for this item and its
+      // copies have landed
+      if (!dead && !__all_sync(0xffffffffu, wait_claimed(tag + s, (int)(w - w0), p.timeout_ns) &&
+                                                mbar_wait(&full[s], ph, p.timeout_ns))) {
+        dead = true;
+        set_status(p.status, kStatusTimeout);
       }
       if (!dead) {
         const uint8_t* slot = smem + (size_t)s * p.slot_bytes;

@@ -267,21 +267,10 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
   int s = grp;
   uint32_t ph = 0;
   for (int n = grp; n < n_items; n += kGroups) {
-    if (kGroups > 1 && !dead && tag[s] != n) {
-      // the slot may still hold an earlier item of another warp: wait until the producer has
-      // claimed it for this one, so that the parity wait below cannot match an older phase
-      const uint64_t w0 = global_ns();
-      while (tag[s] != n) {
-        __nanosleep(32);
-        if (global_ns() - w0 > p.timeout_ns) {
-          dead = true;
-          set_status(p.status, kStatusTimeout);
-          break;
-        }
-      }
-      dead = __any_sync(0xffffffffu, dead);
-    }
-    if (!dead && !__all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.timeout_ns))) {
+    // one vote, in front of which every lane comes: the slot is claimed for this item (where
+    // other warps' items pass through it too) and its copies have landed
+    if (!dead && !__all_sync(0xffffffffu, (kGroups == 1 || wait_claimed(tag + s, n, p.timeout_ns)) &&
+                                              mbar_wait(&full[s], ph, p.timeout_ns))) {
       dead = true;
       set_status(p.status, kStatusTimeout);
     }
