@@ -49,6 +49,10 @@ extern "C" {
 #define SP_CHUNK_MASK_BYTES 1024
 #define SP_CHUNK_ALIGN 16
 
+/* The part of a workspace that must be zero before its first use: its first
+   SP_WORKSPACE_ZERO_BYTES bytes (all of it if it is smaller).  The rest may hold anything. */
+#define SP_WORKSPACE_ZERO_BYTES 65536
+
 typedef enum sp_status {
   SP_OK = 0,
   SP_ERR_INVALID_ARG = 1,   /* null pointer, negative or zero size, bad enum */
@@ -121,8 +125,9 @@ sp_status sp_workspace_size(const sp_matrix* h, int64_t m, size_t* bytes);
  * on chip by their bitmasks; equal to the dense product with the masked weight.
  *   x_dev      [m, K] bf16.      y_dev [m, N] bf16 (fully overwritten).
  *   workspace  device memory of at least sp_workspace_size(h, m) bytes, zero-filled
- *              before its first use; every call leaves it ready for the next one.
- *              Calls that share a workspace must be ordered on one stream.
+ *              before its first use (SP_WORKSPACE_ZERO_BYTES); every call leaves it ready
+ *              for the next one.  Calls that share a workspace must be ordered on one
+ *              stream, and made by one thread at a time: a call may be several launches.
  *   m == 0 returns SP_OK without a launch.  No allocation, no host sync: the call
  *   can be captured in a CUDA graph.  Results are bitwise repeatable for a given
  *   (matrix, m, device). */
@@ -258,6 +263,12 @@ sp_status sp_copy_out(const sp_matrix* h, void* buf_host, size_t buf_cap, uint64
  * Returns SP_ERR_TIMEOUT if a kernel's bounded wait expired since the last
  * check, SP_ERR_CUDA if the stream reported an error, else SP_OK. */
 sp_status sp_check(void* stream);
+
+/* (Library plumbing; no counterpart in the paper.)  The identifier of the graph capture that
+ * `stream` is part of, written to *id: unique in the process, 0 outside a capture.  For
+ * callers that keep a workspace per stream: one that a captured call used belongs to the
+ * graph, which reads it again at each replay.  Host only. */
+sp_status sp_capture_id(void* stream, uint64_t* id);
 
 /* Static English name of a status code (library plumbing; no counterpart in the paper). */
 const char* sp_status_string(sp_status s);

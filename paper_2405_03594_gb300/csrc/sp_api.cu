@@ -298,6 +298,24 @@ sp_status sp_copy_out(const sp_matrix* h, void* buf_host, size_t buf_cap, uint64
   return SP_OK;
 }
 
+sp_status sp_capture_id(void* stream, uint64_t* id) {
+  if (!id) return SP_ERR_INVALID_ARG;
+  *id = 0;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  unsigned long long n = 0;
+  const cudaError_t e = cudaStreamGetCaptureInfo((cudaStream_t)stream, &st, &n);
+  if (e == cudaErrorStreamCaptureImplicit) {  // the legacy stream beside another stream's capture
+    cudaGetLastError();
+    return SP_OK;
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return SP_ERR_CUDA;
+  }
+  if (st == cudaStreamCaptureStatusActive) *id = n;
+  return SP_OK;
+}
+
 sp_status sp_check(void* stream) {
   if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) {
     cudaGetLastError();

@@ -88,9 +88,11 @@ struct LinearParams {
 
 // Workspace layout, fixed per device so that calls with different grids can share it:
 // [arrival counters for up to 2 * kMaxGridPerSm * SMs partial slots][fp32 partials].
-// Every call leaves the counters at zero.
+// Every call leaves the counters at zero; they are the only part that has to be zero before the
+// first call (SP_WORKSPACE_ZERO_BYTES, room for 2048 SMs).
 constexpr int kMaxGridPerSm = 4;
 constexpr int kMaxTokens = 16;  // batch rows per CUDA-core launch (larger batches take several)
+static_assert(SP_WORKSPACE_ZERO_BYTES >= 2 * kMaxGridPerSm * 2048 * sizeof(int), "counters of 2048 SMs");
 inline size_t ws_counter_bytes(int num_sms) {
   return ((size_t)2 * kMaxGridPerSm * num_sms * sizeof(int) + 255) / 256 * 256;
 }

@@ -7,6 +7,7 @@ or PyTorch fallback for any operation here.
 """
 from __future__ import annotations
 
+import collections
 import ctypes
 import os
 import threading
@@ -27,7 +28,7 @@ SP_ERR_UNSUPPORTED = 2
 # every function declared in include/sp.h and include/sp_stack.h
 EXPORTS = ["sp_compress", "sp_decompress", "sp_workspace_size", "sp_linear", "sp_linear_ex", "sp_launch_count",
            "sp_linear_noalloc", "sp_test_expired_wait", "sp_masked_update", "sp_linear_w8a8", "sp_w8a8_workspace_size",
-           "sp_clone", "sp_free", "sp_info", "sp_copy_out", "sp_check", "sp_status_string",
+           "sp_clone", "sp_free", "sp_info", "sp_copy_out", "sp_check", "sp_capture_id", "sp_status_string",
            "sp_copy_columns", "sp_residual_add", "sp_mul_halves", "sp_mul_pairs", "sp_chain_workspace_size",
            "sp_chain_run", "sp_linear_epi"]
 
@@ -82,6 +83,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.sp_info.argtypes = [P, ctypes.POINTER(SpInfo)]
     lib.sp_copy_out.argtypes = [P, P, SZ, P, SZ]
     lib.sp_check.argtypes = [P]
+    lib.sp_capture_id.argtypes = [P, ctypes.POINTER(ctypes.c_uint64)]
     lib.sp_copy_columns.argtypes = [P, P, I64, I64, I64, I64, P]
     lib.sp_residual_add.argtypes = [P, P, P, I64, I64, P]
     lib.sp_mul_halves.argtypes = [P, P, I64, I64, P]
@@ -194,7 +196,7 @@ class SparseMatrix:
         if out is None:
             out = torch.empty((m, self.n), dtype=torch.bfloat16, device=x.device)
         if workspace is None:
-            workspace = workspace_for(self.workspace_size(m), x.device)
+            workspace = workspace_for(self.workspace_size(m), x.device, stream)
         _check(_lib.sp_linear_ex(self._h, x.data_ptr(), m, out.data_ptr(), workspace.data_ptr(), workspace.numel(),
                                  PATHS[path], _stream(stream, self.device)), "sp_linear")
         return out
@@ -210,7 +212,7 @@ class SparseMatrix:
         ny = self.n // 2 if epilogue == "pair_product" else self.n
         assert out.dtype == torch.bfloat16 and out.shape == (m, ny) and out.is_contiguous()
         if workspace is None:
-            workspace = workspace_for(self.workspace_size(m), x.device)
+            workspace = workspace_for(self.workspace_size(m), x.device, stream)
         code = _lib.sp_linear_epi(self._h, x.data_ptr(), m, out.data_ptr(), EPILOGUES[epilogue],
                                   0 if r is None else r.data_ptr(), workspace.data_ptr(), workspace.numel(),
                                   _stream(stream, self.device))
@@ -251,7 +253,7 @@ class SparseMatrix:
         if out is None:
             out = torch.empty((m, self.n), dtype=torch.bfloat16, device=qx.device)
         if workspace is None:
-            workspace = workspace_for(self.w8a8_workspace_size(m), qx.device)
+            workspace = workspace_for(self.w8a8_workspace_size(m), qx.device, stream)
         _check(_lib.sp_linear_w8a8(self._h, _ptr(qx), _ptr(sx), m, _ptr(out), _ptr(workspace), workspace.numel(),
                                    _stream(stream, self.device)), "sp_linear_w8a8")
         return out
@@ -315,18 +317,57 @@ def compress(w: torch.Tensor, mask: torch.Tensor, scale: torch.Tensor | None = N
     return SparseMatrix(h)
 
 
-_ws_cache: dict = {}
+# ------------------------------------------------------------------ default workspaces
+_WS_ZERO_BYTES = 65536  # SP_WORKSPACE_ZERO_BYTES
+_WS_KEPT = 8            # streams whose workspace a thread keeps
 
 
-def workspace_for(nbytes: int, device) -> torch.Tensor:
-    """A zero-filled workspace of at least nbytes on `device`, shared by calls on one stream."""
+class _Workspaces(threading.local):
+    def __init__(self):
+        self.kept = collections.OrderedDict()  # (device, stream, capture) -> tensor, oldest use first
+        self.capture = ctypes.c_uint64()
+
+
+_workspaces = _Workspaces()
+
+
+def workspace_for(nbytes: int, device, stream=None) -> torch.Tensor:
+    """A workspace of at least nbytes on `device` for calls on `stream` (default: the current one).
+
+    Calls that share a workspace must be ordered on one stream and come from one thread, so each
+    thread keeps one per stream (of the last eight), grown as needed.  It is allocated on that stream:
+    when it is outgrown, dropped or its thread ends, its memory is reused in that stream's order
+    only.  Calls captured into a graph share a workspace of that capture, allocated from the
+    graph's memory like every tensor made while torch.cuda.graph captures, since replays may
+    overlap other work and outlive what this thread keeps."""
     dev = torch.device(device)
-    key = dev.index if dev.index is not None else torch.cuda.current_device()
-    ws = _ws_cache.get(key)
-    if ws is None or ws.numel() < max(nbytes, 1):
-        ws = torch.zeros(max(nbytes, 256), dtype=torch.uint8, device=torch.device("cuda", key))
-        _ws_cache[key] = ws
+    index = dev.index if dev.index is not None else torch.cuda.current_device()
+    handle = _stream(stream, index)
+    local = _workspaces
+    _check(_lib.sp_capture_id(handle, ctypes.byref(local.capture)), "sp_capture_id")
+    key = (index, handle, local.capture.value)
+    kept = local.kept
+    ws = kept.get(key)
+    if ws is not None and ws.numel() >= nbytes:
+        kept.move_to_end(key)
+        return ws
+    for k in [k for k in kept if k[2] not in (0, key[2])]:  # of captures that have ended
+        del kept[k]
+    kept.pop(key, None)
+    if stream is not None and not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(handle, device=index)
+    with torch.cuda.device(index), torch.cuda.stream(stream):  # stream None: the current one
+        ws = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=torch.device("cuda", index))
+        ws[:_WS_ZERO_BYTES].zero_()
+    kept[key] = ws
+    while len(kept) > _WS_KEPT:
+        kept.popitem(last=False)
     return ws
+
+
+def release_workspaces() -> None:
+    """Drop the default workspaces that the calling thread keeps."""
+    _workspaces.kept.clear()
 
 
 def copy_columns(out: torch.Tensor, inp: torch.Tensor, col0: int, stream=None) -> torch.Tensor:
