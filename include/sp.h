@@ -62,7 +62,7 @@ typedef enum sp_status {
   SP_ERR_OUT_OF_MEMORY = 5, /* the allocator returned NULL */
   SP_ERR_TIMEOUT = 6,       /* a bounded device wait expired (reported by sp_check) */
   SP_ERR_BAD_HANDLE = 7,    /* not a live sp_matrix */
-  SP_ERR_WORKSPACE = 8      /* workspace missing or smaller than sp_workspace_size() */
+  SP_ERR_WORKSPACE = 8      /* workspace missing or too small (sp_workspace_size) */
 } sp_status;
 
 typedef enum sp_dtype { SP_BF16 = 0, SP_INT8 = 1 } sp_dtype;
@@ -117,7 +117,9 @@ sp_status sp_decompress(const sp_matrix* h, void* w_out_dev, void* stream);
 
 /* Bytes of device workspace that sp_linear needs for a batch of m rows (its split-K scratch, or
  * for large batches room for the expanded matrix, 2 bytes per weight; library plumbing with no
- * counterpart in the paper), written to *bytes (0 for m == 0).  Host only.  SP_ERR_INVALID_ARG for m < 0 or a null `bytes`. */
+ * counterpart in the paper), written to *bytes (0 for m == 0).  A workspace without that room
+ * still serves a large batch, more slowly, if it holds the split-K scratch (at most 262,144 bytes
+ * per SM and a few KB).  Host only.  SP_ERR_INVALID_ARG for m < 0 or a null `bytes`. */
 sp_status sp_workspace_size(const sp_matrix* h, int64_t m, size_t* bytes);
 
 /* y = x . (W o Mask)^T, FP32 accumulation, bf16 output (round to nearest even): the sparse
@@ -130,7 +132,7 @@ sp_status sp_workspace_size(const sp_matrix* h, int64_t m, size_t* bytes);
  *              stream, and made by one thread at a time: a call may be several launches.
  *   m == 0 returns SP_OK without a launch.  No allocation, no host sync: the call
  *   can be captured in a CUDA graph.  Results are bitwise repeatable for a given
- *   (matrix, m, device). */
+ *   (matrix, m, device), and workspaces that all hold sp_workspace_size bytes. */
 sp_status sp_linear(const sp_matrix* h, const void* x_dev, int64_t m, void* y_dev, void* workspace_dev,
                     size_t workspace_bytes, void* stream);
 

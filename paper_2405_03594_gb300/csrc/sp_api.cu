@@ -29,14 +29,32 @@ bool live(const sp_matrix* h) { return h && h->magic == SP_MAGIC; }
 constexpr int64_t kCudaCoreMaxM_bf16 = 10;
 constexpr int64_t kCudaCoreMaxM_int8 = 13;
 
+// What the kernels that make one launch need between them.
+size_t workspace_one_launch(const sp_matrix* h, int64_t m) {
+  return std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m));
+}
+
 // Workspace of the documented contract, whatever kernel runs a batch of m rows.  One size serves
 // every batch of more than 240 rows (the widest token tile), on either tensor-core route.
 size_t workspace_bytes(const sp_matrix* h, int64_t m) {
-  const size_t b = std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m));
+  const size_t b = workspace_one_launch(h, m);
   const int64_t md = m > 240 ? 257 : m;  // as uses_dense has it from there on
   return uses_dense(h, md) ? std::max(b, workspace_bytes_dense(h, md)) : b;
 }
 
+}  // namespace
+
+// What a linear call that is given `have` bytes uses of them: the documented size, or, where that
+// includes room for the expanded matrix and there is less, what the one-launch kernels need (they
+// then run the batch).  0: too little for either.
+size_t workspace_used(const sp_matrix* h, int64_t m, size_t have) {
+  const size_t full = workspace_bytes(h, m);
+  if (have >= full) return full;
+  const size_t one = workspace_one_launch(h, m);
+  return have >= one ? one : 0;
+}
+
+namespace {
 bool uses_tensor_cores(const sp_matrix* h, int64_t m, sp_path path) {
   const int64_t cc_max = h->esize == 1 ? kCudaCoreMaxM_int8 : kCudaCoreMaxM_bf16;
   return path == SP_PATH_TENSOR_CORE || (path == SP_PATH_AUTO && m > cc_max);
@@ -134,8 +152,7 @@ sp_status sp_linear_ex(const sp_matrix* h, const void* x_dev, int64_t m, void* y
     return SP_ERR_CUDA;
   }
   if (dev != h->device) return SP_ERR_INVALID_ARG;
-  if (!workspace_dev || workspace_bytes < sp::workspace_bytes(h, m))
-    return SP_ERR_WORKSPACE;
+  if (!workspace_dev || workspace_used(h, m, workspace_bytes) == 0) return SP_ERR_WORKSPACE;
   if (uses_tensor_cores(h, m, path))
     return launch_linear_tc(h, static_cast<const uint16_t*>(x_dev), m, static_cast<uint16_t*>(y_dev), workspace_dev,
                             workspace_bytes, (cudaStream_t)stream);
@@ -162,8 +179,7 @@ sp_status sp_linear_epi(const sp_matrix* h, const void* x_dev, int64_t m, void* 
     return SP_ERR_CUDA;
   }
   if (dev != h->device) return SP_ERR_INVALID_ARG;
-  if (!workspace_dev || workspace_bytes < sp::workspace_bytes(h, m))
-    return SP_ERR_WORKSPACE;
+  if (!workspace_dev || workspace_used(h, m, workspace_bytes) == 0) return SP_ERR_WORKSPACE;
   if (uses_tensor_cores(h, m, SP_PATH_AUTO)) return SP_ERR_UNSUPPORTED;
   return launch_linear_cc(h, static_cast<const uint16_t*>(x_dev), m, static_cast<uint16_t*>(y_dev), workspace_dev,
                           workspace_bytes, (cudaStream_t)stream, true, 0, epilogue,
@@ -204,8 +220,7 @@ sp_status sp_test_expired_wait(const sp_matrix* h, const void* x_dev, int64_t m,
     return SP_ERR_CUDA;
   }
   if (dev != h->device) return SP_ERR_INVALID_ARG;
-  if (!workspace_dev || workspace_bytes < sp::workspace_bytes(h, m))
-    return SP_ERR_WORKSPACE;
+  if (!workspace_dev || workspace_used(h, m, workspace_bytes) == 0) return SP_ERR_WORKSPACE;
   return launch_linear_cc(h, static_cast<const uint16_t*>(x_dev), m, static_cast<uint16_t*>(y_dev), workspace_dev,
                           workspace_bytes, (cudaStream_t)stream, true, (uint64_t)wait_ms * 1000000ull);
 }

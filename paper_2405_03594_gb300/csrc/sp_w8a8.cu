@@ -84,11 +84,11 @@ extern "C" sp_status sp_linear_w8a8(const sp_matrix* h, const int8_t* qx_dev, co
     return SP_ERR_CUDA;
   }
   if (dev != h->device) return SP_ERR_INVALID_ARG;
-  size_t lin = 0, need = 0;
-  sp_status st = sp_workspace_size(h, m, &lin);
-  if (st == SP_OK) st = sp_w8a8_workspace_size(h, m, &need);
-  if (st != SP_OK) return st;
-  if (!workspace_dev || workspace_bytes < need) return SP_ERR_WORKSPACE;
+  // the widened x lies behind what the linear uses of the rest (workspace_used)
+  const size_t xb = round256((size_t)m * (size_t)h->K * 2);
+  const size_t have = workspace_bytes > xb ? (workspace_bytes - xb) / 256 * 256 : 0;
+  const size_t lin = workspace_used(h, m, have);
+  if (!workspace_dev || lin == 0) return SP_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace_dev);
   uint4* x = reinterpret_cast<uint4*>(ws + round256(lin));
   const int64_t k8 = h->K / 8;  // K % 8 == 0 (checked at compression)

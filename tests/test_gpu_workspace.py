@@ -139,3 +139,53 @@ def test_a_graph_keeps_its_workspace(oracle, M):
         assert np.array_equal(gu.bf16_bits_from_dev(y), want)
         assert np.array_equal(gu.bf16_bits_from_dev(yb), want_big)
         assert np.array_equal(gu.bf16_bits_from_dev(yo), want_big)
+
+
+@pytest.mark.parametrize("int8", [False, True])
+@pytest.mark.parametrize("N,K,M", [(4096, 4096, 33), (9000, 2056, 300)])
+def test_large_batch_without_room_for_the_expanded_matrix(oracle, N, K, M, int8):
+    """A workspace of the one-launch kernels' size is accepted, and one byte less is not."""
+    import torch
+
+    from paper_2405_03594_gb300 import sp
+
+    g = np.random.default_rng(N + M)
+    mask = (g.random((N, K)) < 0.3).astype(np.uint8)
+    x = synth.bf16_from_f32(g.integers(-2, 3, size=(M, K)).astype(np.float32))
+    rows = np.unique(np.concatenate([[0, N - 1], g.choice(N, 200, replace=False)]))
+    if int8:
+        v = g.integers(-128, 128, size=(N, K)).astype(np.int8)
+        s = np.exp2(g.integers(-3, 4, size=N)).astype(np.float32)
+        h = sp.compress(gu.i8_to_dev(v), gu.u8_to_dev(mask), gu.f32_to_dev(s))
+        ref = oracle.linear_int8(x, v[rows], mask[rows], s[rows])
+    else:
+        v = synth.bf16_from_f32(g.integers(-4, 5, size=(N, K)).astype(np.float32))
+        h = sp.compress(gu.bf16_to_dev(v), gu.u8_to_dev(mask))
+        ref = oracle.linear_bf16(x, v[rows], mask[rows])
+    want = synth.bf16_from_f32(ref.astype(np.float32))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    counters = (32 * sms + 255) // 256 * 256
+    ntok = min(256, (M + 15) // 16 * 16)
+    # split-K partials of 128 rows: two per CTA, of 16 tokens on up to four CTAs per SM (its first
+    # 16 rows' kernels) or of the token tile on one
+    size = max(h.workspace_size(1), counters + 2 * sms * 128 * ntok * 4)
+    assert size < h.workspace_size(M)
+    xd = gu.bf16_to_dev(x)
+    ws = torch.zeros(size, dtype=torch.uint8, device=gu.dev())
+    y = torch.full((M, N), float("nan"), dtype=torch.bfloat16, device=gu.dev())
+    h.linear(xd, out=y, workspace=ws)
+    sp.check()
+    assert not ws[:counters].any()
+    assert np.array_equal(gu.bf16_bits_from_dev(y)[:, rows], want)
+    with pytest.raises(sp.SpError) as e:
+        h.linear(xd, out=y, workspace=ws[:size - 1])
+    assert e.value.code == 8
+    if int8:  # activations that are whole numbers widen exactly with unit scales
+        xb = (M * K * 2 + 255) // 256 * 256
+        ws = torch.zeros((size + 255) // 256 * 256 + xb, dtype=torch.uint8, device=gu.dev())
+        assert ws.numel() < h.w8a8_workspace_size(M)
+        y.fill_(float("nan"))
+        qx = gu.i8_to_dev(synth.bf16_to_f32(x).astype(np.int8))
+        h.linear_w8a8(qx, gu.f32_to_dev(np.ones(M, dtype=np.float32)), out=y, workspace=ws)
+        sp.check()
+        assert np.array_equal(gu.bf16_bits_from_dev(y)[:, rows], want)
