@@ -34,12 +34,15 @@ size_t workspace_one_launch(const sp_matrix* h, int64_t m) {
   return std::max(workspace_bytes_cc(h, m), workspace_bytes_tc(h, m));
 }
 
-// Workspace of the documented contract, whatever kernel runs a batch of m rows.  One size serves
-// every batch of more than 240 rows (the widest token tile), on either tensor-core route.
+// Workspace of the documented contract, whatever kernel runs a batch of m rows.  Where the matrix
+// is expanded first, the partials of linear_tc_kernel, whose grid grows with the batch up to an SM
+// each, are not part of it, so one size serves every batch of more than 240 rows (the widest token
+// tile).  A matrix of fewer than 16 chunks stays on linear_tc_kernel, and its size grows with the
+// batch until the grid fills the SMs.
 size_t workspace_bytes(const sp_matrix* h, int64_t m) {
-  const size_t b = workspace_one_launch(h, m);
   const int64_t md = m > 240 ? 257 : m;  // as uses_dense has it from there on
-  return uses_dense(h, md) ? std::max(b, workspace_bytes_dense(h, md)) : b;
+  return uses_dense(h, md) ? std::max(workspace_bytes_cc(h, m), workspace_bytes_dense(h, md))
+                           : workspace_one_launch(h, m);
 }
 
 }  // namespace

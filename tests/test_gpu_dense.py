@@ -54,10 +54,10 @@ def test_integer_sums_bit_exact(oracle, N, K, M, int8):
 
 
 @pytest.mark.parametrize("int8", [False, True])
-@pytest.mark.parametrize("N,K", [(8960, 8192), (2048, 1024)])
+@pytest.mark.parametrize("N,K", [(8960, 8192), (2048, 1024), (1024, 1200), (1024, 512), (256, 512)])
 def test_one_workspace_size_above_240_rows(N, K, int8):
     """A workspace sized for one batch of more than 240 rows serves every other one, and none
-    of fewer rows needs more."""
+    of fewer rows needs more: matrices of 16 chunks and more, of fewer chunks than SMs too."""
     from paper_2405_03594_gb300 import sp
 
     g = np.random.default_rng(9)
@@ -65,6 +65,42 @@ def test_one_workspace_size_above_240_rows(N, K, int8):
     size = h.workspace_size(241)
     assert {h.workspace_size(m) for m in (249, 250, 256, 257, 2048, (1 << 24) + 1)} == {size}
     assert max(h.workspace_size(m) for m in (1, 2, 16, 32, 33, 100, 200, 240)) <= size
+
+
+def test_workspace_sized_at_241_rows_runs_2048(oracle):
+    """64 chunks, fewer than SMs: linear_tc_kernel would need more at 2048 rows than at 241."""
+    import torch
+
+    from paper_2405_03594_gb300 import sp
+
+    g = np.random.default_rng(3)
+    (W, mask, _), h = _matrix(sp, 1024, 512, False, g)
+    x = synth.bf16_from_f32(g.integers(-2, 3, size=(2048, 512)).astype(np.float32))
+    ws = torch.zeros(h.workspace_size(241), dtype=torch.uint8, device=gu.dev())
+    y = h.linear(gu.bf16_to_dev(x), workspace=ws)
+    sp.check()
+    ref = oracle.linear_bf16(np.ascontiguousarray(x[::64]), W, mask)
+    assert np.array_equal(gu.bf16_bits_from_dev(y)[::64], synth.bf16_from_f32(ref.astype(np.float32)))
+
+
+def test_fewer_than_16_chunks_need_more_for_more_rows(oracle):
+    """15 chunks stay on linear_tc_kernel: each batch's own size serves it and every smaller one."""
+    import torch
+
+    from paper_2405_03594_gb300 import sp
+
+    g = np.random.default_rng(4)
+    (W, mask, _), h = _matrix(sp, 384, 320, False, g)
+    Ms = (1, 32, 33, 240, 241, 300, 2048, 5000)
+    sizes = [h.workspace_size(m) for m in Ms]
+    assert sizes == sorted(sizes) and h.launch_count(2048) == 1
+    x = synth.bf16_from_f32(g.integers(-2, 3, size=(2048, 320)).astype(np.float32))
+    for M in (241, 2048):
+        ws = torch.zeros(h.workspace_size(M), dtype=torch.uint8, device=gu.dev())
+        y = h.linear(gu.bf16_to_dev(x[:M]), workspace=ws)
+        sp.check()
+        ref = oracle.linear_bf16(np.ascontiguousarray(x[:M:48]), W, mask)
+        assert np.array_equal(gu.bf16_bits_from_dev(y)[::48], synth.bf16_from_f32(ref.astype(np.float32)))
 
 
 def test_update_then_large_batch_on_one_stream(oracle):
