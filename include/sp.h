@@ -130,6 +130,9 @@ sp_status sp_workspace_size(const sp_matrix* h, int64_t m, size_t* bytes);
  *              before its first use (SP_WORKSPACE_ZERO_BYTES); every call leaves it ready
  *              for the next one.  Calls that share a workspace must be ordered on one
  *              stream, and made by one thread at a time: a call may be several launches.
+ *   An infinite or NaN x[m, k] reaches only the outputs whose row keeps column k on the
+ *   CUDA-core family.  On the tensor-core family a dropped column counts as +0 times x, as in
+ *   the dense product, so it makes NaN in every output of row m.
  *   m == 0 returns SP_OK without a launch.  No allocation, no host sync: the call
  *   can be captured in a CUDA graph.  Results are bitwise repeatable for a given
  *   (matrix, m, device), and workspaces that all hold sp_workspace_size bytes. */

@@ -305,6 +305,19 @@ __device__ __forceinline__ void st_cluster_f32(uint32_t caddr, float v) {
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
+// The same barrier; whether v holds in any of its threads.
+__device__ __forceinline__ bool named_bar_or(int id, int nthreads, bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %3, 0;\n\t"
+      "bar.red.or.pred q, %1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(id), "r"(nthreads), "r"((uint32_t)v)
+      : "memory");
+  return r != 0;
+}
 __device__ __forceinline__ void set_status(int* status, int code) {
   if (status) atomicCAS(status, kStatusOk, code);
 }
@@ -330,8 +343,9 @@ int cc_kernel_kind(const sp_matrix* h, int64_t M);  // 0 thread-per-row, 1 warp-
 // the expansion is worth sharing across a wider token tile.
 constexpr int kMmaMaxRows = 32;
 bool uses_mma(const sp_matrix* h, int64_t M);  // the rule: that kernel is the faster one, and fits
+// kept_only: the CUDA-core family's results for an infinite or NaN x (a dropped column takes no part)
 sp_status launch_linear_mma(const sp_matrix* h, const uint16_t* x, int64_t M, uint16_t* y, cudaStream_t stream,
-                            int32_t epi, const uint16_t* r);
+                            int32_t epi, const uint16_t* r, bool kept_only);
 sp_status launch_linear_tc(const sp_matrix* h, const uint16_t* x, int64_t M, uint16_t* y, void* ws, size_t ws_bytes,
                            cudaStream_t stream);
 size_t workspace_bytes_tc(const sp_matrix* h, int64_t M);

@@ -978,7 +978,7 @@ sp_status launch_linear_cc(const sp_matrix* h, const uint16_t* x, int64_t M, uin
   for (int64_t m0 = 0; m0 < M; m0 += kMaxTokens) {
     const int Mt = (int)std::min<int64_t>(kMaxTokens, M - m0);
     if (on_mma(Mt)) {
-      const sp_status st = launch_linear_mma(h, x + m0 * h->K, Mt, y + m0 * ldy, stream, epi, r);
+      const sp_status st = launch_linear_mma(h, x + m0 * h->K, Mt, y + m0 * ldy, stream, epi, r, true);
       if (st != SP_OK) return st;
       continue;
     }

@@ -54,16 +54,18 @@ struct MmaParams {
   const uint64_t* off;
   const uint64_t* qidx;
   const float* scale;  // INT8 only
+  const uint16_t* x;
   uint16_t* y;
   const uint16_t* r;   // SP_EPI_RESIDUAL
   int* status;
-  int64_t N, C;        // output rows; chunks
+  int64_t N, K, C;     // output rows; columns; chunks
   int32_t T, M;
   int32_t cluster;     // CTAs per row block
   int32_t slots;
   uint32_t chunk_region, ring_off, tab_off, bar_off, lut_off, rx_off;
   int32_t epi;
   int32_t early;       // release the next launch as soon as this one's inputs are ready
+  int32_t kept_only;   // x of a dropped column takes no part, infinite or NaN either
   uint64_t timeout_ns;
 };
 
@@ -147,6 +149,95 @@ __device__ __forceinline__ void write_one(const MmaParams& p, int64_t n, int m, 
           bf16_bits_to_float(p.r[n]));
     else
       *yp = (uint16_t)b;
+  }
+}
+
+// Row rr of row block seg times tokens m, m + step, .. (four, those past M repeat m) over the kept
+// columns of K-tiles [t0, t1), from global memory: the kept-weight walk's sums.  All lanes of a warp
+// call it together with consecutive rows.  Bound by the latency of its loads.
+template <int ES>
+__device__ __forceinline__ float4 kept_sums(const MmaParams& p, int64_t seg, int t0, int t1, int rr, int m, int step) {
+  const int lane = rr & 31;
+  const uint16_t* x[4];
+  float sum[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    x[j] = p.x + (int64_t)(m + j * step < p.M ? m + j * step : m) * p.K;
+    sum[j] = 0.f;
+  }
+  for (int t = t0; t < t1; ++t) {
+    const int64_t c = seg * p.T + t;
+    const uint8_t* chunk = p.buf + p.off[c];
+    uint64_t mk = reinterpret_cast<const uint64_t*>(chunk)[rr];
+    const int pc = __popcll(mk);
+    int e = pc;  // kept entries of the warp's rows up to this one
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, e, d);
+      if (lane >= d) e += u;
+    }
+    e -= pc;
+    if (rr >= 32) e += (int)((p.qidx[c] >> (16 * (rr / 32 - 1))) & 0xffffu);
+    const uint8_t* val = chunk + kMaskBytes + (int64_t)e * ES;
+    while (mk) {
+      float w[4], v[4][4];
+      bool on[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        on[i] = mk != 0;
+        if (on[i]) {
+          const int64_t k = (int64_t)kTileK * t + __ffsll((long long)mk) - 1;
+          w[i] = ES == 2 ? bf16_bits_to_float(*reinterpret_cast<const uint16_t*>(val))
+                         : (float)*reinterpret_cast<const int8_t*>(val);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            v[i][j] = bf16_bits_to_float(__ldcg(reinterpret_cast<const unsigned short*>(x[j] + k)));
+          val += ES;
+          mk &= mk - 1;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (on[i]) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) sum[j] = fmaf(w[i], v[i][j], sum[j]);
+        }
+    }
+    __syncwarp();
+  }
+  return make_float4(sum[0], sum[1], sum[2], sum[3]);
+}
+
+// The matrix product multiplies a dropped column's +0 with x, which for an infinite or NaN x makes
+// every row of the token NaN; the walk, which runs the CUDA-core family's other batches, never
+// touches a dropped column.  For that family the CTA's sums ([groups][M][kRows] in comb) that are
+// not finite are therefore taken again over the kept columns, by the thread that reads them next:
+// row rr of tokens m0, m0 + step, ..  Finite inputs pay a multiply-add per sum and a vote, where the
+// sums are read anyway (gate/up at M = 4 27.6 -> 27.7 us; tested in the registers before they meet
+// in shared memory 27.95), and the call keeps the rare code's registers out of the kernel's.  With
+// a NaN in one of 3 to 10 tokens o takes 100 us, gate/up 115 to 140.
+template <int ES>
+__device__ __noinline__ void redo_sums(const MmaParams& p, float* comb, int64_t seg, int t0, int t1, int rr, int m0,
+                                       int step, int groups) {
+  const int M = p.M;
+  for (int m = m0; m < M; m += 4 * step) {
+    bool redo[4];
+    bool any = false;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int mj = m + j * step;
+      float z = 0.f;
+      for (int q = 0; mj < M && q < groups; ++q) z = fmaf(comb[(q * M + mj) * kRows + rr], 0.f, z);
+      any |= redo[j] = z != z;
+    }
+    if (!__any_sync(0xffffffffu, any)) continue;
+    const float4 k = kept_sums<ES>(p, seg, t0, t1, rr, m, step);
+    const float kj[4] = {k.x, k.y, k.z, k.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (redo[j]) {
+        for (int q = 0; q < groups; ++q) comb[(q * M + m + j * step) * kRows + rr] = q == 0 ? kj[j] : 0.f;
+      }
   }
 }
 
@@ -369,21 +460,28 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
   const int rr = tid % kRows, m0 = tid / kRows;
   const int64_t row = seg * kRows + rr;
   const float sc = (ES == 1 && row < p.N) ? p.scale[row] : 1.f;
-  if (p.cluster == 1) {
-    for (int m = m0; m < M; m += kStep) {
-      float v = comb[m * kRows + rr];
-#pragma unroll
-      for (int q = 1; q < kGroups; ++q) v += comb[(q * M + m) * kRows + rr];
-      write_one(p, row, m, v, sc);
-    }
-    return;
-  }
   auto cta_sum = [&](int m) {
     float v = comb[m * kRows + rr];
 #pragma unroll
     for (int q = 1; q < kGroups; ++q) v += comb[(q * M + m) * kRows + rr];
     return v;
   };
+  // z: 0 times each of the warp's sums, added up; not 0 if one of them is not finite.  The CUDA-core
+  // family's batches (at most 16 rows a launch) then take those sums again.
+  auto redo = [&](float z, int groups) {
+    if (NT > 2 || !__any_sync(0xffffffffu, p.kept_only && z != 0.f)) return false;
+    redo_sums<ES>(p, comb, seg, t0, t1, rr, m0, kStep, groups);
+    return true;
+  };
+  float z = 0.f;
+  if (p.cluster == 1) {
+    if (NT <= 2 && p.kept_only) {
+      for (int m = m0; m < M; m += kStep) z = fmaf(cta_sum(m), 0.f, z);
+      redo(z, kGroups);
+    }
+    for (int m = m0; m < M; m += kStep) write_one(p, row, m, cta_sum(m), sc);
+    return;
+  }
   if constexpr (kPush) {
     // Few tokens: rank m % S owns token m, and every CTA stores its sum of it straight into the
     // owner's receive area ([tokens owned][S][kRows] floats, apart from the ring, which the
@@ -396,8 +494,16 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
     const int S = p.cluster;
     const uint32_t rx = smem_u32(smem + p.rx_off) + 4u * (uint32_t)(rank * kRows + rr);
     cluster_wait();
-    for (int m = m0; m < M; m += kStep)
-      st_cluster_f32(cluster_map(rx + 4u * (uint32_t)(m / S * S * kRows), (uint32_t)(m % S)), cta_sum(m));
+    auto push = [&](int m, float v) {
+      st_cluster_f32(cluster_map(rx + 4u * (uint32_t)(m / S * S * kRows), (uint32_t)(m % S)), v);
+    };
+    for (int m = m0; m < M; m += kStep) {
+      const float v = cta_sum(m);
+      push(m, v);
+      z = fmaf(v, 0.f, z);
+    }
+    if (redo(z, kGroups))
+      for (int m = m0; m < M; m += kStep) push(m, cta_sum(m));
     cluster_arrive_release();
     cluster_wait();
     const float* got = reinterpret_cast<const float*>(smem + p.rx_off) + rr;
@@ -409,8 +515,13 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
     }
     return;
   }
-  if constexpr (kGroups > 1) {
-    for (int m = m0; m < M; m += kStep) comb[m * kRows + rr] = cta_sum(m);
+  if (kGroups > 1 || (NT <= 2 && p.kept_only)) {
+    for (int m = m0; m < M; m += kStep) {
+      const float v = cta_sum(m);
+      if (kGroups > 1) comb[m * kRows + rr] = v;
+      z = fmaf(v, 0.f, z);
+    }
+    redo(z, 1);
   }
   cluster_sync_all();
   const uint32_t mine = smem_u32(comb) + 4u * (uint32_t)rr;
@@ -637,7 +748,7 @@ bool uses_mma(const sp_matrix* h, int64_t M) {
 }
 
 sp_status launch_linear_mma(const sp_matrix* h, const uint16_t* x, int64_t M, uint16_t* y, cudaStream_t stream,
-                            int32_t epi, const uint16_t* r) {
+                            int32_t epi, const uint16_t* r, bool kept_only) {
   if (M < 1 || M > kMmaMaxRows) return SP_ERR_UNSUPPORTED;
   MmaChoice c;
   MmaPlan pl;
@@ -650,10 +761,12 @@ sp_status launch_linear_mma(const sp_matrix* h, const uint16_t* x, int64_t M, ui
   p.off = h->d_off;
   p.qidx = h->d_qidx;
   p.scale = h->d_scale;
+  p.x = x;
   p.y = y;
   p.r = r;
   p.status = device_status_ptr();
   p.N = h->N;
+  p.K = h->K;
   p.C = (int64_t)h->RB * h->T;
   p.T = h->T;
   p.M = (int32_t)M;
@@ -666,6 +779,7 @@ sp_status launch_linear_mma(const sp_matrix* h, const uint16_t* x, int64_t M, ui
   p.lut_off = pl.lut_off;
   p.rx_off = pl.rx_off;
   p.epi = epi;
+  p.kept_only = kept_only ? 1 : 0;
   p.early = overlaps((int64_t)h->RB * pl.cluster, (int64_t)c.occ * h->num_sms) ? 1 : 0;
   p.timeout_ns = wait_timeout_ns();
   // x [M, K] bf16, box = 64 columns x 8 NT tokens, 128-byte swizzle; rows past M and columns
