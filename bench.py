@@ -373,7 +373,9 @@ def dense_section(host, xs, results, Ms):
 KERNEL_SOURCES = {
     "linear_ccw_kernel": ("sp_linear_cc.cu", "sp_cc_common.cuh", "sp_internal.cuh"),
     "linear_cc_kernel": ("sp_linear_cc.cu", "sp_cc_common.cuh", "sp_internal.cuh"),
+    "linear_mma_kernel": ("sp_linear_mma.cu", "sp_expand.cuh", "sp_internal.cuh"),
     "linear_tc_kernel": ("sp_linear_tc.cu", "sp_expand.cuh", "sp_tcgen05.cuh", "sp_internal.cuh"),
+    "expand_kernel + dense_kernel": ("sp_linear_dense.cu", "sp_expand.cuh", "sp_tcgen05.cuh", "sp_internal.cuh"),
     "chain_kernel": ("sp_chain.cu", "sp_cc_common.cuh", "sp_internal.cuh"),
 }
 
@@ -986,17 +988,17 @@ def run_single(args):
 
 def square_section(args) -> dict:
     """The 12288 x 12288 sparse matmul against sparsity (the scaling example of Sec. 2.3, there
-    on a CS-3; here on the tensor-core kernel): x [2048, 12288] bf16, per-row magnitude masks at
+    on a CS-3; here the matrix is expanded and multiplied densely): x [2048, 12288] bf16, per-row magnitude masks at
     0, 10, ..., 90 %, y = x . (W o M)^T.  Per sparsity the launch time, its speedup over the 0 %
-    matrix through the same kernel, the ideal 1 / (1 - s), and the speedup over the dense cuBLAS
+    matrix through the same kernels, the ideal 1 / (1 - s), and the speedup over the dense cuBLAS
     GEMM of the same shape.  Parity of this shape is checked by the GPU tests.  A failure is
     reported in the section instead of ending the run."""
     import torch
 
     from paper_2405_03594_gb300 import sp, synth
 
-    out = {"what": "12288 x 12288, M = 2048, tensor-core kernel, per-row magnitude masks", "N": 12288, "K": 12288,
-           "M": 2048, "kernel": "linear_tc_kernel", "points": {}}
+    out = {"what": "12288 x 12288, M = 2048, tensor-core family, per-row magnitude masks", "N": 12288, "K": 12288,
+           "M": 2048, "kernel": None, "points": {}}
     try:
         dev = torch.device("cuda", 0)
         N = K = 12288
@@ -1027,6 +1029,7 @@ def square_section(args) -> dict:
             mask = synth.magnitude_mask(W, pct)
             h = sp.compress(Wd, torch.from_numpy(mask).to(dev))
             ws = torch.zeros(max(h.workspace_size(M), 256), dtype=torch.uint8, device=dev)
+            out["kernel"] = h.kernel_name(M, "tensor_core")
             us = timed(lambda: h.linear(xd, out=y, workspace=ws, path="tensor_core"))
             sp.check()
             base = us if base is None else base

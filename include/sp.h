@@ -143,26 +143,33 @@ sp_status sp_linear(const sp_matrix* h, const void* x_dev, int64_t m, void* y_de
 sp_status sp_linear_ex(const sp_matrix* h, const void* x_dev, int64_t m, void* y_dev, void* workspace_dev,
                        size_t workspace_bytes, sp_path path, void* stream);
 
-/* Kernels that sp_linear_ex can launch (reported by sp_launch_count): the family's choice for
-   the batch.  Within either family, batches of up to 32 rows mostly run on linear_mma_kernel
-   (warp-level matrix instructions on chunks expanded in registers), which is the faster one
-   there; the report stays the family's. */
+/* Kernels that sp_linear_ex can launch (reported by sp_launch_count).  Within either family,
+   batches of up to 32 rows mostly run on linear_mma_kernel, which is the faster one there. */
 enum {
   SP_KERNEL_NONE = 0,
   SP_KERNEL_CC_THREAD_PER_ROW = 1,  /* linear_cc_kernel: four warps share a chunk, thread = row */
   SP_KERNEL_CC_WARP_PER_CHUNK = 2,  /* linear_ccw_kernel (M <= 4): a warp per chunk, lane = 4 rows */
-  SP_KERNEL_TENSOR_CORE = 3         /* linear_tc_kernel; expand_kernel and dense_kernel for 2 launches */
+  SP_KERNEL_TENSOR_CORE = 3,        /* linear_tc_kernel: chunks expanded into tensor memory */
+  SP_KERNEL_WARP_MMA = 4,           /* linear_mma_kernel: chunks expanded in registers, warp-level MMA */
+  SP_KERNEL_EXPAND_DENSE = 5        /* expand_kernel, then dense_kernel: the matrix expanded first */
 };
 
 /* (Library plumbing; no counterpart in the paper.)  Number of kernel launches that
  * sp_linear_ex(h, x, m, y, ws, ws_bytes, path, stream)
  * makes, written to *launches: 0 for m == 0, one per 16 batch rows on the CUDA-core
  * family, one on the tensor-core family, or two where it expands the matrix first (large
- * batches); if `kernel` is not null, the SP_KERNEL_* value
- * of the kernel used for the first 16 rows (or all rows) goes there.  For callers that
- * count launches or label profiles.  Host only: no GPU work.  SP_ERR_BAD_HANDLE for a
+ * batches, in a workspace of sp_workspace_size bytes); if `kernel` is not null, the SP_KERNEL_*
+ * value of the kernel used for the first 16 rows (CUDA-core family) or all rows goes there.  For
+ * callers that count launches or label profiles.  Host only: no GPU work.  SP_ERR_BAD_HANDLE for a
  * dead handle, SP_ERR_INVALID_ARG for m < 0, an unknown path or a null `launches`. */
 sp_status sp_launch_count(const sp_matrix* h, int64_t m, sp_path path, int64_t* launches, int32_t* kernel);
+
+/* (Library plumbing; no counterpart in the paper.)  The kernel family that sp_linear_ex takes for
+ * m rows on `path`, SP_PATH_CUDA_CORE or SP_PATH_TENSOR_CORE, written to *family.  The family,
+ * not the kernel, says which batches sp_linear_epi accepts and what an infinite or NaN x reaches.
+ * Host only.  SP_ERR_BAD_HANDLE for a dead handle, SP_ERR_INVALID_ARG for m < 0, an unknown path
+ * or a null `family`. */
+sp_status sp_kernel_family(const sp_matrix* h, int64_t m, sp_path path, int32_t* family);
 
 /* sp_linear for callers that may not allocate device memory (the paper has no
  * counterpart; this is a deployment convenience).  Some callers receive only their

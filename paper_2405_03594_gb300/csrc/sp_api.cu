@@ -198,11 +198,21 @@ sp_status sp_launch_count(const sp_matrix* h, int64_t m, sp_path path, int64_t* 
   if (kernel) {
     if (m == 0)
       *kernel = SP_KERNEL_NONE;
+    else if (uses_mma(h, tc ? m : std::min<int64_t>(m, kMaxTokens)))
+      *kernel = SP_KERNEL_WARP_MMA;
     else if (tc)
-      *kernel = SP_KERNEL_TENSOR_CORE;
+      *kernel = uses_dense(h, m) ? SP_KERNEL_EXPAND_DENSE : SP_KERNEL_TENSOR_CORE;
     else
       *kernel = cc_kernel_kind(h, m) == 1 ? SP_KERNEL_CC_WARP_PER_CHUNK : SP_KERNEL_CC_THREAD_PER_ROW;
   }
+  return SP_OK;
+}
+
+sp_status sp_kernel_family(const sp_matrix* h, int64_t m, sp_path path, int32_t* family) {
+  if (!live(h)) return SP_ERR_BAD_HANDLE;
+  if (m < 0 || !family || (path != SP_PATH_AUTO && path != SP_PATH_CUDA_CORE && path != SP_PATH_TENSOR_CORE))
+    return SP_ERR_INVALID_ARG;
+  *family = uses_tensor_cores(h, m, path) ? SP_PATH_TENSOR_CORE : SP_PATH_CUDA_CORE;
   return SP_OK;
 }
 

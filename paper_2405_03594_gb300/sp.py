@@ -27,13 +27,15 @@ STATUS = {
 SP_ERR_UNSUPPORTED = 2
 # every function declared in include/sp.h and include/sp_stack.h
 EXPORTS = ["sp_compress", "sp_decompress", "sp_workspace_size", "sp_linear", "sp_linear_ex", "sp_launch_count",
+           "sp_kernel_family",
            "sp_linear_noalloc", "sp_test_expired_wait", "sp_masked_update", "sp_linear_w8a8", "sp_w8a8_workspace_size",
            "sp_clone", "sp_free", "sp_info", "sp_copy_out", "sp_check", "sp_capture_id", "sp_status_string",
            "sp_copy_columns", "sp_residual_add", "sp_mul_halves", "sp_mul_pairs", "sp_chain_workspace_size",
            "sp_chain_run", "sp_linear_epi"]
 
 
-KERNELS = {0: "", 1: "linear_cc_kernel", 2: "linear_ccw_kernel", 3: "linear_tc_kernel"}  # SP_KERNEL_*
+KERNELS = {0: "", 1: "linear_cc_kernel", 2: "linear_ccw_kernel", 3: "linear_tc_kernel", 4: "linear_mma_kernel",
+           5: "expand_kernel + dense_kernel"}  # SP_KERNEL_*
 
 
 class SpError(RuntimeError):
@@ -73,6 +75,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.sp_linear.argtypes = [P, P, I64, P, P, SZ, P]
     lib.sp_linear_ex.argtypes = [P, P, I64, P, P, SZ, ctypes.c_int, P]
     lib.sp_launch_count.argtypes = [P, I64, ctypes.c_int, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int32)]
+    lib.sp_kernel_family.argtypes = [P, I64, ctypes.c_int, ctypes.POINTER(ctypes.c_int32)]
     lib.sp_linear_noalloc.argtypes = [P, P, I64, P, P]
     lib.sp_test_expired_wait.argtypes = [P, P, I64, P, P, SZ, ctypes.c_uint32, P]
     lib.sp_masked_update.argtypes = [P, P, ctypes.c_float, P]
@@ -183,10 +186,18 @@ class SparseMatrix:
         return int(n.value)
 
     def kernel_name(self, m: int, path: str = "auto") -> str:
-        """Name of the kernel that linear() runs for a batch of m rows on `path`."""
+        """Name of the kernel that linear() runs for a batch of m rows on `path` (for more than
+        16 rows on the CUDA-core family, for the first 16)."""
         n, k = ctypes.c_int64(), ctypes.c_int32()
         _check(_lib.sp_launch_count(self._h, m, PATHS[path], ctypes.byref(n), ctypes.byref(k)), "sp_launch_count")
         return KERNELS[k.value]
+
+    def kernel_family(self, m: int, path: str = "auto") -> str:
+        """The kernel family that linear() takes for m rows on `path`: "cuda_core" (whose batches
+        linear_epi() accepts) or "tensor_core"."""
+        f = ctypes.c_int32()
+        _check(_lib.sp_kernel_family(self._h, m, PATHS[path], ctypes.byref(f)), "sp_kernel_family")
+        return "tensor_core" if f.value == PATHS["tensor_core"] else "cuda_core"
 
     def linear(self, x: torch.Tensor, out: torch.Tensor | None = None, workspace: torch.Tensor | None = None,
                path: str = "auto", stream=None) -> torch.Tensor:
@@ -205,7 +216,7 @@ class SparseMatrix:
                    workspace: torch.Tensor | None = None, stream=None) -> bool:
         """sp_linear_epi: out = epilogue(x . (W o Mask)^T) with "store", "residual" (out updated
         in place with the bf16 vector r [N]) or "pair_product" (out [m, N/2]).  Returns False,
-        launching nothing, where the batch would run on the tensor-core kernel (the caller
+        launching nothing, where linear() takes the tensor-core family (kernel_family; the caller
         then uses linear() and the glue call)."""
         assert x.dtype == torch.bfloat16 and x.dim() == 2 and x.shape[1] == self.k and x.is_contiguous()
         m = x.shape[0]

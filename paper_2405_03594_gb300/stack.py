@@ -128,7 +128,7 @@ class LinearStack:
 
     def fuses(self, M: int) -> bool:
         """Whether a step of M rows folds the residual adds and gate * up into the linears."""
-        return self.fused and all(self.mats[n][0].kernel_name(M) != "linear_tc_kernel" for n in SHAPES)
+        return self.fused and all(self.mats[n][0].kernel_family(M) == "cuda_core" for n in SHAPES)
 
     def launches_per_step(self, M: int, reset: bool = True) -> int:
         """libsp kernels per step: the four sparse linears (as many launches as the library

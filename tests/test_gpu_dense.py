@@ -33,7 +33,7 @@ def test_integer_sums_bit_exact(oracle, N, K, M, int8):
 
     g = np.random.default_rng(N * K + M)
     (v, mask, s), h = _matrix(sp, N, K, int8, g)
-    assert h.launch_count(M) == 2  # the expansion and the product
+    assert h.launch_count(M) == 2 and h.kernel_name(M) == "expand_kernel + dense_kernel"
     x = synth.bf16_from_f32(g.integers(-2, 3, size=(M, K)).astype(np.float32))
     ws = torch.zeros(h.workspace_size(M), dtype=torch.uint8, device=gu.dev())
     y = torch.full((M, N), float("nan"), dtype=torch.bfloat16, device=gu.dev())

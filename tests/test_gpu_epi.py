@@ -88,7 +88,7 @@ def test_tensor_core_batches_are_declined(sp):
     M = 64
     x = gu.bf16_to_dev(synth.activations(M, 4096, np.random.default_rng(0)))
     ws = torch.zeros(max(h.workspace_size(M), 256), dtype=torch.uint8, device="cuda")
-    assert h.kernel_name(M) == "linear_tc_kernel"
+    assert h.kernel_family(M) == "tensor_core"
     y = torch.full((M, 4096), 7.0, dtype=torch.bfloat16, device="cuda")
     assert not h.linear_epi(x, y, "store", workspace=ws)
     torch.cuda.synchronize()

@@ -274,8 +274,17 @@ def test_launch_count(sp):
     assert h8.launch_count(40, "cuda_core") == 3
     with pytest.raises(sp.SpError):
         h.launch_count(-1)
-    assert h.kernel_name(1) == "linear_ccw_kernel" and h.kernel_name(8) == "linear_cc_kernel"
-    assert h.kernel_name(11) == "linear_tc_kernel" and h.kernel_name(3, "tensor_core") == "linear_tc_kernel"
+    # the kernels that run: the walk for one row, the tcgen05 kernel above 32 rows (12 chunks: too
+    # few to be expanded first), the warp-level matrix kernel between, in either family
+    assert h.kernel_name(1) == "linear_ccw_kernel" and h.kernel_name(8) == "linear_mma_kernel"
+    assert h.kernel_name(11) == "linear_mma_kernel" and h.kernel_name(3, "tensor_core") == "linear_mma_kernel"
+    assert h.kernel_name(40, "cuda_core") == "linear_mma_kernel" and h.kernel_name(33) == "linear_tc_kernel"
+    assert h.kernel_name(0) == "" and h.kernel_name(1, "tensor_core") == "linear_tc_kernel"
+    assert [h.kernel_family(m) for m in (1, 10, 11)] == ["cuda_core", "cuda_core", "tensor_core"]
+    assert [h8.kernel_family(m) for m in (13, 14)] == ["cuda_core", "tensor_core"]
+    assert h.kernel_family(1, "tensor_core") == "tensor_core" and h.kernel_family(40, "cuda_core") == "cuda_core"
+    with pytest.raises(sp.SpError):
+        h.kernel_family(-1)
 
 
 def test_shared_workspace_across_grids(sp, oracle):

@@ -33,6 +33,7 @@ def test_integer_sums_bit_exact(oracle, N, K, M, int8):
         h = sp.compress(gu.bf16_to_dev(W), gu.u8_to_dev(mask))
         ref = oracle.linear_bf16(x, W, mask)
     for path in ("auto", "cuda_core") if M <= 16 else ("auto",):
+        assert h.kernel_name(M, path) == "linear_mma_kernel"
         y = h.linear(gu.bf16_to_dev(x), path=path)
         sp.check()
         assert np.array_equal(gu.bf16_bits_from_dev(y), synth.bf16_from_f32(ref.astype(np.float32))), path
@@ -50,6 +51,7 @@ def test_large_chunks_at_lower_occupancy(oracle, N, K, M, least):
     x = synth.bf16_from_f32(g.integers(-2, 3, size=(M, K)).astype(np.float32))
     W = synth.bf16_from_f32(g.integers(-4, 5, size=(N, K)).astype(np.float32))
     h = sp.compress(gu.bf16_to_dev(W), gu.u8_to_dev(mask))
+    assert h.kernel_name(M) == "linear_mma_kernel"
     y = h.linear(gu.bf16_to_dev(x))
     sp.check()
     ref = oracle.linear_bf16(x, W, mask)
@@ -71,6 +73,8 @@ def test_one_and_two_rows_of_many_int8_weights(oracle, N, K, keep, M):
     s = np.exp2(g.integers(-3, 4, size=N)).astype(np.float32)
     x = synth.bf16_from_f32(g.integers(-2, 3, size=(M, K)).astype(np.float32))
     h = sp.compress(gu.i8_to_dev(q), gu.u8_to_dev(mask), gu.f32_to_dev(s))
+    many = h.info.nnz >= (0.36 if M == 1 else 0.26) * N * K
+    assert (h.kernel_name(M) == "linear_mma_kernel") == many
     ws = torch.zeros(max(h.workspace_size(M), 256), dtype=torch.uint8, device=gu.dev())
     y = h.linear(gu.bf16_to_dev(x), workspace=ws)
     ref = oracle.linear_int8(x, q, mask, s)

@@ -30,7 +30,7 @@ def test_shared_segments_bit_exact(oracle, N, K, Ms, int8):
         h = sp.compress(gu.bf16_to_dev(v), gu.u8_to_dev(mask))
     rows = np.unique(np.concatenate([[0, N - 1], g.choice(N, 200, replace=False)]))
     for M in Ms:
-        assert h.launch_count(M) == 1
+        assert h.launch_count(M) == 1 and h.kernel_name(M) == "linear_tc_kernel"
         x = synth.bf16_from_f32(g.integers(-2, 3, size=(M, K)).astype(np.float32))
         ws = torch.zeros(h.workspace_size(M), dtype=torch.uint8, device=gu.dev())
         ref = oracle.linear_int8(x, v[rows], mask[rows], s[rows]) if int8 else oracle.linear_bf16(x, v[rows], mask[rows])
