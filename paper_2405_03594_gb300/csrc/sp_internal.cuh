@@ -354,6 +354,7 @@ size_t workspace_bytes_tc(const sp_matrix* h, int64_t M);
 bool uses_dense(const sp_matrix* h, int64_t M);  // the rule: that way is the faster one
 size_t workspace_bytes_dense(const sp_matrix* h, int64_t M);
 size_t workspace_used(const sp_matrix* h, int64_t m, size_t have);  // of the bytes a call is given; 0: too few
+// SP_ERR_UNSUPPORTED, with nothing launched, where the device holds no CTA pair of the product
 sp_status launch_linear_dense(const sp_matrix* h, const uint16_t* x, int64_t M, uint16_t* y, void* ws, size_t ws_bytes,
                               cudaStream_t stream);
 sp_status tensor_map_encoder(PFN_cuTensorMapEncodeTiled_v12000* out);  // cuTensorMapEncodeTiled, looked up once

@@ -24,6 +24,7 @@
 #include <cstring>
 
 #include "sp_expand.cuh"
+#include "sp_lookup.h"
 #include "sp_tcgen05.cuh"
 
 namespace sp {
@@ -481,12 +482,11 @@ void plan_items(const sp_matrix* h, int64_t M, int pairs, DenseParams* p) {
   }
 }
 
-// CTA pairs that the device holds at once (0: the kernel cannot run); looked up once per device.
+// CTA pairs that the device, which is current, holds at once; 0: none, or the lookup failed.
 int resident_pairs(int dev) {
-  static std::atomic<int> pairs[kMaxDevices] = {};  // + 1; 0 = not looked up
+  static std::atomic<int> pairs[kMaxDevices] = {};
   if (dev < 0 || dev >= kMaxDevices) return 0;
-  int n = pairs[dev].load(std::memory_order_acquire);
-  if (n == 0) {
+  return kept_or_looked_up(pairs[dev], [] {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2);
     cfg.blockDim = dim3(kDenseThreads);
@@ -498,10 +498,8 @@ int resident_pairs(int dev) {
       cudaGetLastError();
       c = 0;
     }
-    n = c + 1;
-    pairs[dev].store(n, std::memory_order_release);
-  }
-  return n - 1;
+    return c;
+  });
 }
 
 size_t round256(size_t b) { return (b + 255) / 256 * 256; }
@@ -541,7 +539,7 @@ sp_status launch_linear_dense(const sp_matrix* h, const uint16_t* x, int64_t M, 
   sp_status st = tensor_map_encoder(&encode);
   if (st != SP_OK) return st;
   const int pairs = std::min(resident_pairs(h->device), h->num_sms / 2);
-  if (pairs < 1) return SP_ERR_CUDA;
+  if (pairs < 1) return SP_ERR_UNSUPPORTED;  // nothing launched; linear_tc_kernel takes the batch
 
   // the scratch follows the arrival counters, which stay zero for the other kernels
   uint8_t* scratch = static_cast<uint8_t*>(ws) + ws_counter_bytes(h->num_sms);

@@ -618,9 +618,12 @@ size_t workspace_bytes_tc(const sp_matrix* h, int64_t M) {
 sp_status launch_linear_tc(const sp_matrix* h, const uint16_t* x, int64_t M, uint16_t* y, void* ws, size_t ws_bytes,
                            cudaStream_t stream) {
   if (uses_mma(h, M)) return launch_linear_mma(h, x, M, y, stream, 0, nullptr, false);
-  // a workspace without room for the expanded matrix keeps the batch on this kernel
-  if (uses_dense(h, M) && ws_bytes >= workspace_bytes_dense(h, M))
-    return launch_linear_dense(h, x, M, y, ws, ws_bytes, stream);
+  // a workspace without room for the expanded matrix keeps the batch on this kernel, as does a
+  // device that holds no CTA pair of the product
+  if (uses_dense(h, M) && ws_bytes >= workspace_bytes_dense(h, M)) {
+    const sp_status st = launch_linear_dense(h, x, M, y, ws, ws_bytes, stream);
+    if (st != SP_ERR_UNSUPPORTED) return st;
+  }
   if (!ws || ws_bytes < workspace_bytes_tc(h, M)) return SP_ERR_WORKSPACE;
   if (M > ((int64_t)1 << 31) / kMaxNtok) return SP_ERR_UNSUPPORTED;
   PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
