@@ -9,9 +9,9 @@
 // memory on one CTA per SM, whatever the tokens.  Here a warp expands 16 columns of two rows per lane
 // directly into the A registers of mma.sync m16n8k16 (bf16, FP32 accumulation), so the cost
 // of a chunk hardly depends on M: four matrix instructions per 16 rows and 8 tokens beside
-// ~290 instructions of expansion.  What bounds it is shared memory: ~530 wavefronts per chunk
-// (predicated two-byte value loads at 1.6 each), 62 % of the peak rate over a gate/up launch
-// (ncu), the rest being launch latency and tail.  Measured at 70 %, bf16, graphs of launches on
+// ~290 instructions of expansion.  What takes most of its time is shared memory: ~520 wavefronts
+// per chunk (predicated two-byte value loads at 1.6 each), 62 % of the peak rate over a gate/up
+// launch (ncu), the rest being launch latency and tail.  Measured at 70 %, bf16, graphs of launches on
 // matrices beyond L2, before / here: gate/up 32.2 / 28.1 us at M = 3, 48.7 / 28.4 at M = 5,
 // 61.6 / 31.5 at M = 10, 46.4 / 32.1 at M = 16, 47.2 / 40.9 at M = 32; o 15.3 / 8.8, 18.2 / 9.6,
 // 20.9 / 9.8, 23.4 / 12.8 at M = 5, 10, 16, 32; INT8 gate/up 54 / 30.8 at M = 5, 55.5 / 35.0 at
@@ -215,11 +215,13 @@ __device__ __forceinline__ float4 kept_sums(const MmaParams& p, int64_t seg, int
 // touches a dropped column.  For that family the CTA's sums ([groups][M][kRows] in comb) that are
 // not finite are therefore taken again over the kept columns, by the thread that reads them next:
 // row rr of tokens m0, m0 + step, ..  Finite inputs pay a multiply-add per sum and a vote, where the
-// sums are read anyway (gate/up at M = 4 27.6 -> 27.7 us; tested in the registers before they meet
-// in shared memory 27.95), and the call keeps the rare code's registers out of the kernel's.  With
-// a NaN in one of 3 to 10 tokens o takes 100 us, gate/up 115 to 140.
+// sums are read anyway: gate/up at M = 4 27.64 -> 27.69 us, a captured step of four layers at
+// M = 4 304.9 -> 307.3.  In line, and only in the forms that need it: a call, taken or not, costs
+// every launch ~0.2 us (the step 309.6; at 16 rows, which never take it, 375.2 -> 379); tested in the
+// registers, before the sums meet in shared memory, gate/up took 27.95.  With a NaN in one of 3 to
+// 10 tokens o takes 100 us, gate/up 110 to 136.
 template <int ES>
-__device__ __noinline__ void redo_sums(const MmaParams& p, float* comb, int64_t seg, int t0, int t1, int rr, int m0,
+__device__ __forceinline__ void redo_sums(const MmaParams& p, float* comb, int64_t seg, int t0, int t1, int rr, int m0,
                                        int step, int groups) {
   const int M = p.M;
   for (int m = m0; m < M; m += 4 * step) {
@@ -243,7 +245,9 @@ __device__ __noinline__ void redo_sums(const MmaParams& p, float* comb, int64_t 
   }
 }
 
-template <int NT, int ES, int RW, int CW, int OCC>
+// KO: the batch may be the CUDA-core family's (p.kept_only says), whose sums that are not finite are
+// taken again.
+template <int NT, int ES, int RW, int CW, int OCC, bool KO>
 __global__ void __launch_bounds__((CW + 1) * 32, OCC)
     linear_mma_kernel(const __grid_constant__ MmaParams p, const __grid_constant__ CUtensorMap tmap_x) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -471,13 +475,13 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
   // z: 0 times each of the warp's sums, added up; not 0 if one of them is not finite.  The CUDA-core
   // family's batches (at most 16 rows a launch) then take those sums again.
   auto redo = [&](float z, int groups) {
-    if (NT > 2 || !__any_sync(0xffffffffu, p.kept_only && z != 0.f)) return false;
+    if (!KO || !__any_sync(0xffffffffu, p.kept_only && z != 0.f)) return false;
     redo_sums<ES>(p, comb, seg, t0, t1, rr, m0, kStep, groups);
     return true;
   };
   float z = 0.f;
   if (p.cluster == 1) {
-    if (NT <= 2 && p.kept_only) {
+    if (KO && p.kept_only) {
       for (int m = m0; m < M; m += kStep) z = fmaf(cta_sum(m), 0.f, z);
       redo(z, kGroups);
     }
@@ -517,7 +521,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
     }
     return;
   }
-  if (kGroups > 1 || (NT <= 2 && p.kept_only)) {
+  if (kGroups > 1 || (KO && p.kept_only)) {
     for (int m = m0; m < M; m += kStep) {
       const float v = cta_sum(m);
       if (kGroups > 1) comb[m * kRows + rr] = v;
@@ -537,10 +541,10 @@ __global__ void __launch_bounds__((CW + 1) * 32, OCC)
 }
 
 // ------------------------------------------------------------------ host side
-template <int NT, int ES, int RW, int CW, int OCC>
+template <int NT, int ES, int RW, int CW, int OCC, bool KO>
 sp_status launch(const sp_matrix* h, const MmaParams& p, const CUtensorMap& map, const MmaPlan& pl,
                  cudaStream_t stream, bool pdl) {
-  auto kern = linear_mma_kernel<NT, ES, RW, CW, OCC>;
+  auto kern = linear_mma_kernel<NT, ES, RW, CW, OCC, KO>;
   static bool configured[kMaxDevices] = {};
   const int dev = h->device;
   if (dev < 0 || dev >= kMaxDevices) return SP_ERR_UNSUPPORTED;
@@ -577,13 +581,16 @@ template <int ES>
 sp_status dispatch(const sp_matrix* h, const MmaParams& p, const CUtensorMap& map, const MmaPlan& pl,
                    const MmaChoice& c, cudaStream_t stream, bool pdl) {
   if (c.nt == 1)
-    return c.cw == 4 ? launch<1, ES, 64, 4, 6>(h, p, map, pl, stream, pdl)
-                     : launch<1, ES, 64, 8, 3>(h, p, map, pl, stream, pdl);
+    return c.cw == 4 ? launch<1, ES, 64, 4, 6, true>(h, p, map, pl, stream, pdl)
+                     : launch<1, ES, 64, 8, 3, true>(h, p, map, pl, stream, pdl);
+  if (c.nt == 2 && p.kept_only)
+    return c.cw == 4 ? launch<2, ES, 32, 4, 5, true>(h, p, map, pl, stream, pdl)
+                     : launch<2, ES, 64, 8, 2, true>(h, p, map, pl, stream, pdl);
   if (c.nt == 2)
-    return c.cw == 4 ? launch<2, ES, 32, 4, 5>(h, p, map, pl, stream, pdl)
-                     : launch<2, ES, 64, 8, 2>(h, p, map, pl, stream, pdl);
-  return c.cw == 4 ? launch<4, ES, 32, 4, 4>(h, p, map, pl, stream, pdl)
-                   : launch<4, ES, 32, 8, 2>(h, p, map, pl, stream, pdl);
+    return c.cw == 4 ? launch<2, ES, 32, 4, 5, false>(h, p, map, pl, stream, pdl)
+                     : launch<2, ES, 64, 8, 2, false>(h, p, map, pl, stream, pdl);
+  return c.cw == 4 ? launch<4, ES, 32, 4, 4, false>(h, p, map, pl, stream, pdl)
+                   : launch<4, ES, 32, 8, 2, false>(h, p, map, pl, stream, pdl);
 }
 
 }  // namespace
@@ -594,7 +601,7 @@ sp_status dispatch(const sp_matrix* h, const MmaParams& p, const CUtensorMap& ma
 // INT8, walk / here: M = 2 at 50 % 592 / 334 us, 60 % 396 / 334, 70 % 350 / 332, 80 % 299 / 331;
 // M = 1 (the o linear, 14 chunks per SM, on the walk) at 50 % 383 / 321, at 60 % 341 / 321, at 70 %
 // 299 / 321.  bf16 at M = 2: 364 / 370, 327 / 350, 295 / 319, 260 / 294; at M = 1 357 / 389,
-// 307 / 359, 263 / 321, 224 / 298.
+// 307 / 359, 263 / 321, 224 / 298.  The lines on the kept share come from that stack alone.
 bool uses_mma(const sp_matrix* h, int64_t M) {
   if (M < 1 || M > kMmaMaxRows || (M == 1 && !large(h))) return false;
   if (M == 1 || (M == 2 && large(h))) {
