@@ -101,7 +101,8 @@ typedef void (*sp_free_fn)(void* ptr, void* ctx);
  *              a masked-out nonzero is dropped.
  *   scale_dev  [N] fp32 per-row scales for SP_INT8 (copied); must be NULL for SP_BF16.
  *   N, K       N >= 1, K >= 1, K % 8 == 0 (SP_ERR_UNSUPPORTED otherwise).
- * Synchronises `stream` once (the total size sizes the buffer).  On success *out
+ * Synchronises `stream` twice: for the total size, which sizes the buffer, and at its end, so
+ * that the inputs and its scratch are free.  On success *out
  * is a new handle owning its device buffers; on error *out is NULL and nothing
  * is leaked.  Inputs are only read and may be freed once the call returns. */
 sp_status sp_compress(const void* w_dev, const uint8_t* mask_dev, int64_t n, int64_t k, sp_dtype dtype,

@@ -25,7 +25,8 @@ bool live(const sp_matrix* h) { return h && h->magic == SP_MAGIC; }
 // Largest batch that the CUDA-core family takes under SP_PATH_AUTO, and that sp_linear_epi
 // accepts; larger batches go to the tensor-core family.  The line was the crossover of
 // linear_cc_kernel and linear_tc_kernel; both families now run linear_mma_kernel around it, so
-// it only says up to which batch the epilogues of sp_chain_epilogue are available.
+// it only says up to which batch the epilogues of sp_chain_epilogue are available, and what an
+// infinite or NaN x reaches (include/sp.h).
 constexpr int64_t kCudaCoreMaxM_bf16 = 10;
 constexpr int64_t kCudaCoreMaxM_int8 = 13;
 

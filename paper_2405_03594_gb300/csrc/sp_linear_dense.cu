@@ -513,7 +513,9 @@ size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 // token tile (q/k/v, 6144 chunks, 41.3 / 31.8 at 64, 49.8 / 48.5 at 256; gate/up, 11008, 76.5 / 42.0
 // and 82.4 / 61.9; two tiles 94 / 120 at 384).  INT8, which linear_tc_kernel expands slower: down
 // 37.5 / 39.7 at 64, q/k/v 41.9 / 41.7 at 128, 14336 x 4096 (7168 chunks) 51.4 / 50.8 at 192, gate/up
-// 82.9 / 67.5 at 256.  A matrix of a few chunks keeps the one launch.
+// 82.9 / 67.5 at 256.  A matrix of a few chunks keeps the one launch.  The lines go by the chunk
+// count alone and hold for 50 to 80 %; on unpruned rows, where linear_tc_kernel's value loads
+// meet in one bank, this way would win far earlier (gate/up at 256: 104 / 368).
 bool uses_dense(const sp_matrix* h, int64_t M) {
   const int64_t C = (int64_t)h->RB * h->T, rows = (int64_t)h->RB * kRows;
   if (C < 16 || M > (int64_t)1 << 24 || (int64_t)h->T * rows >= (int64_t)1 << 31) return false;

@@ -5,11 +5,13 @@
 // griddepcontrol.wait (which returns once every earlier grid of the stream has completed).
 // At M = 1 a glue kernel releases the next launch at once, so the next linear's CTAs
 // become resident and copy weights while the glue runs; at M > 1 the release comes with
-// the glue's exit.  Measured on GB300 (graph of the 32-layer step, 70%): early release
-// 450 / 1277 tok/s at M = 1 / 4 (bf16), release at exit 432 / 1358, no PDL 446 / 1144;
-// the M = 1 linears run six CTAs per SM and gain from early residency, the four-per-SM
-// M > 1 linears lose by it (their CTAs land unevenly in the slots the previous linear's
-// tail leaves).
+// the glue's exit.  Measured on GB300 at M = 1 (graph of the 32-layer step, 70 %, bf16, glue
+// after every linear): early release 450 tok/s, at exit 432, without PDL 446.  At M > 1 the
+// linears around the glue are linear_mma_kernel's; graph of a four-layer step, 70 %, bf16, us
+// at exit / early: M = 2 296.6 / 292.9, 4 309 / 307, 8 319 / 316, where one copy of v per layer
+// is all the glue there is, but 379 / 423 at 16 and 453 / 530 at 32, with four glue kernels per
+// layer (INT8 342 / 338, 338 / 336, 350 / 346, 409 / 449, 475 / 552): the next linear's CTAs then
+// land unevenly in the slots that the previous one's tail leaves.
 #include "../../include/sp_stack.h"
 #include "sp_internal.cuh"
 

@@ -19,8 +19,9 @@
 // costs ~0.3 us of the SM's issue slots against 0.75 us of its share of the HBM rate.
 // Measured, 4096 x 11008 at 70 %, the step and the weight read back dense: 105.5 us with the
 // gradient in two-column pieces and the values read and written in global memory, 64.3 us so.
-// Five CTAs per SM (48 registers, 12 bytes of spills) against four: 22016 x 4096 78.5 -> 74.2 us
-// (480 MB, 6.5 TB/s); 512 threads per CTA with half the rows each 87.
+// Five CTAs per SM (48 registers, 12 bytes of spills) against four: 22016 x 4096 78.5 -> 74.2 us;
+// 512 threads per CTA with half the rows each 87.  That moves 480 MB, the whole gradient among
+// them (6.5 TB/s); 460 MB would do, since 6 % of its 32-byte sectors hold no kept weight (6.2).
 #include "sp_internal.cuh"
 
 namespace sp {

@@ -12,6 +12,8 @@
 // griddepcontrol.wait (every earlier grid of the stream has completed), and it releases the
 // linear that follows at once for one-row batches (whose six-CTA launch then copies its
 // weights while the widening runs) and at its exit otherwise, as the stack's glue kernels do.
+// Calls back to back, 70 %, us at exit / early: gate/up 33.3 / 32.8 at M = 2, 39.7 / 38.0 at 16,
+// 52.2 / 50.9 at 64, but q/k/v 24.9 / 26.5 to 27.7 at 16 and 28.7 / 32.8 to 34.4 at 32.
 #include <algorithm>
 
 #include "sp_internal.cuh"
